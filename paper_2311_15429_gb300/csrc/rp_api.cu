@@ -19,12 +19,6 @@
 
 #include "rp_ctx.h"
 
-namespace rp {
-size_t smem_direct(int max_nlag);
-int direct_blocks(long long n);
-cudaError_t open_direct_smem_limit(int max_optin);
-}  // namespace rp
-
 using namespace rp;
 
 namespace {
@@ -1163,7 +1157,7 @@ rp_status rp_finalize(rp_ctx *ctx)
             P.nx_s = S.n[0]; P.ny_s = S.n[1]; P.nz_s = S.n[2];
             P.n_s = S.N;
             P.dx = T.o[0] - S.o[0]; P.dy = T.o[1] - S.o[1]; P.dz = T.o[2] - S.o[2];
-            P.hs = (float)S.h;
+            P.hs = S.h;
             P.vol = (float)(S.h * S.h * S.h);
             P.is_self = t == s;
             P.self_w = t == s ? (float)(cube_average_constant() * S.h * S.h) : 0.0f;
@@ -1177,7 +1171,10 @@ rp_status rp_finalize(rp_ctx *ctx)
         if (D.p1 > D.p0) {
             D.block0 = ctx->dir_blocks;
             D.accumulate = tgt_fft[t];
-            ctx->dir_blocks += direct_blocks(T.N);
+            bool shared = false;
+            D.groups = direct_groups(T.n[0], T.h, cdt, &shared);
+            D.shared = shared ? 1 : 0;
+            ctx->dir_blocks += direct_blocks(T.n, D.groups);
             ctx->dtg.push_back(D);
         }
     }
@@ -1187,7 +1184,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         for (int t = 0; t < nd; ++t)
             for (int s = 0; s < nd; ++s)
                 rdepth[s] = std::max(rdepth[s], ctx->pairs[(size_t)t * nd + s].lag_hi + 1 + (ctx->overlap ? 1 : 0));
-    ctx->smem_dir = smem_direct(max_nlag);
+    ctx->dir_nlag = max_nlag;
     ctx->raw_block0.assign(nd + 1, 0);
     for (int d = 0; d < nd; ++d) {
         int nb = 0;
@@ -1237,7 +1234,9 @@ rp_status rp_finalize(rp_ctx *ctx)
     RP_CUDA(ctx, cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     ctx->smem_optin = max_optin;
     {
-        const size_t need = std::max({ctx->smem_plane, ctx->smem_col, ctx->smem_mac, ctx->smem_inv, ctx->smem_dir});
+        const size_t need = std::max({ctx->smem_plane, ctx->smem_col, ctx->smem_mac, ctx->smem_inv});
+        if (max_nlag > kDirMaxLags)
+            return fail(ctx, RP_ERR_UNSUPPORTED, "direct pair lag window above " + std::to_string(kDirMaxLags) + " steps");
         if (need > (size_t)max_optin)
             return fail(ctx, RP_ERR_UNSUPPORTED, "kernel shared memory " + std::to_string(need) +
                                                      " B exceeds the device limit " + std::to_string(max_optin));
@@ -1278,6 +1277,31 @@ rp_status rp_finalize(rp_ctx *ctx)
     for (DirectPair &P : ctx->dpairs) {
         P.raw = ctx->raw[P.src].ring;
         P.depth = ctx->raw[P.src].depth;
+    }
+    if (!ctx->dtg.empty()) {
+        // the direct sums' sources in parts, summed afterwards from a workspace;
+        // in one part, with no workspace, under a device budget or where the
+        // device has no room for it
+        long long least = 0, nodes = 0;
+        for (const DirectPair &P : ctx->dpairs) least = least ? std::min(least, P.n_s) : P.n_s;
+        for (const DirectTarget &D : ctx->dtg) nodes += D.n;
+        ctx->dir_splits = ctx->cfg.device_budget > 0 ? 1 : direct_splits(ctx->dir_blocks, least);
+        if (ctx->dir_splits > 1) {
+            st = dev_alloc(ctx, &ctx->dir_part, (size_t)(4 * nodes * ctx->dir_splits));
+            if (st == RP_ERR_OOM) {
+                cudaGetLastError();
+                ctx->dir_splits = 1;
+            } else if (st) {
+                return st;
+            }
+        }
+        if (ctx->dir_splits > 1) {
+            long long at = 0;
+            for (DirectTarget &D : ctx->dtg) {
+                D.part0 = at;
+                at += 4 * D.n * ctx->dir_splits;
+            }
+        }
     }
 
     // ---- kernel spectra (FP64 on the host, stored FP32), built in parallel;
@@ -1927,10 +1951,11 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
             return st;
     }
     if (!ctx->dtg.empty()) {
-        const float inv_cdt = (float)(1.0 / (ctx->cfg.c * ctx->cfg.dt));
+        const double inv_cdt = 1.0 / (ctx->cfg.c * ctx->cfg.dt);
         if ((st = timed_launch(ctx, RP_K_DIRECT, "direct sum", [&] {
-                 return launch_direct(ctx->d_dtg, (int)ctx->dtg.size(), ctx->d_dpairs, out, ctx->dir_blocks,
-                                      ctx->smem_dir, kstep, clamp, inv_cdt, inv_c, ctx->stream);
+                 return launch_direct(ctx->d_dtg, (int)ctx->dtg.size(), ctx->d_dpairs, out, ctx->dir_part,
+                                      ctx->dir_splits, ctx->dir_blocks, ctx->dir_nlag, kstep, clamp, inv_cdt, inv_c,
+                                      ctx->stream);
              })))
             return st;
     }

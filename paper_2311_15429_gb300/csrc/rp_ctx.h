@@ -162,7 +162,9 @@ struct rp_ctx {
     std::vector<RawRing> raw;
     std::vector<int> raw_block0;                     // [ndom + 1], blocks of k_ring_push
     int plane_blocks = 0, col_blocks = 0, mac_blocks = 0, invp_blocks = 0, dir_blocks = 0;
-    size_t smem_plane = 0, smem_col = 0, smem_mac = 0, smem_inv = 0, smem_dir = 0;
+    size_t smem_plane = 0, smem_col = 0, smem_mac = 0, smem_inv = 0;
+    int dir_nlag = 0, dir_splits = 1;                // direct sums: longest lag window, parts of the sources
+    float *dir_part = nullptr;                       // their workspace (more than one part)
     bool fwd_tile[7] = {}, inv_tile[7] = {};            // plane-pass form per class (index by class_slot)
     size_t smem_plane_cls[7] = {}, smem_inv_cls[7] = {}; // their shared memory per launch
     int max_lag = 0, raw_depth = 0, spec_depth = 0;

@@ -5,9 +5,30 @@
 //   S(l - tau) = (1 - w) S_{l-m} + w S_{l-m-1},  m = floor(tau), w = tau - m
 //
 // (Eq. 8 with the hat interpolation of Eq. 7; at R = 0 of the self pair the
-// cell-averaged weight C h^2 at lag 0).  One thread per target node; a block
-// stages kDirTile source nodes with their samples for the pair's lag window
-// in shared memory; each of the four sums is Kahan-compensated in FP32.
+// cell-averaged weight C h^2 at lag 0).
+//
+// Bound by instruction issue and by what shared memory returns to registers
+// (128 B/clk per SM, broadcasts included), about 1e9 node pairs per step of
+// two 32^3 grids against some 5 MB of samples.  What that asks for:
+//   * a thread owns four target nodes and walks the sources with the geometry
+//     of two in packed FP32 pairs (add/mul/fma.f32x2), and floor by a
+//     round-down addition of 2^23 (no conversion);
+//   * the samples lie as 16 bytes (rho, Jx, Jy, Jz) per [lag][source]; four
+//     neighbours along x no farther apart than light goes in a step (SHARED)
+//     see at most two lag intervals, so three samples serve all four.  Where
+//     they are farther apart, or rows so short that groups of four would be
+//     mostly padding, each target loads its own two (direct_groups);
+//   * the eight warps of a block share 128 targets and divide a staged tile of
+//     sources, and blockIdx.y divides the sources again (direct_splits), so
+//     that small grids fill the chip too; k_direct_sum adds the parts in order;
+//   * a warp adds runs of up to 8 sources in plain FP32 and each run's sum
+//     Kahan-compensated to its total (the node itself, whose weight outgrows
+//     its neighbours', on its own).
+// 32^3 (h 0.25) and 27^3 (h 0.3), both cross pairs, 1.29e9 node pairs a step:
+// 7060 us with one thread per target, scalar samples and a Kahan addition per
+// term; 2300 us with two targets per thread and a sample pair each; 1730 us in
+// this form (55 % of issue slots; neither more warps nor scalar arithmetic in
+// place of the packed changes that).
 #include <cuda_runtime.h>
 
 #include "rp_internal.h"
@@ -16,8 +37,12 @@ namespace rp {
 
 namespace {
 
-constexpr int kDirThreads = 128;
-constexpr int kDirTile = 64;
+constexpr int kDirThreads = 256;
+constexpr int kDirWarps = kDirThreads / 32;
+constexpr int kDirOwn = 4;                  // target nodes of a thread
+constexpr int kDirTargets = 32 * kDirOwn;   // target places of a block
+constexpr int kDirRun = 8;                  // sources added before a compensated addition
+constexpr float kFloorShift = 8388608.0f;   // 2^23: x + 2^23 rounded down holds floor(x) in its low bits
 
 __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x)
 {
@@ -27,98 +52,350 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x)
     sum = t;
 }
 
-__global__ void __launch_bounds__(kDirThreads) k_direct(const DirectTarget *__restrict__ tgts, int ntgt,
-                                                          const DirectPair *__restrict__ pairs, OutPtrs out,
-                                                          long long step, int clamp, float inv_cdt, float inv_c)
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 4-byte asynchronous global -> shared copy
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
+                 : "memory");
+}
+
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+
+__device__ __forceinline__ void direct_add(float4 &sum, float4 &comp, float2 a, float2 b)
+{
+    kahan_add(sum.x, comp.x, a.x);
+    kahan_add(sum.y, comp.y, a.y);
+    kahan_add(sum.z, comp.z, b.x);
+    kahan_add(sum.w, comp.w, b.y);
+}
+
+// Shared memory of a block: two buffers of the sample rows (lag_lo twice,
+// lag_lo + 1, ..., lag_hi three times; the repeats serve a tau that rounding
+// put just outside the window) and the tile's negated source positions, the
+// threads' compensated sums (touched once a run), and the rows' offsets into
+// the raw ring.
+__host__ __device__ constexpr int direct_buf_elems(int nlag, int tile) { return (nlag + 3) * (tile + 1) + tile; }
+constexpr int kDirSums = 2 * kDirWarps * kDirTargets;   // float4
+
+// A thread's targets, in packed pairs, relative to the source origin (in units of c dt).
+struct DirectNodes {
+    float2 x[2], y[2], z[2];
+};
+
+// A run of a staged tile: sources jj = j .. j + count - 1 onto the thread's
+// targets, which SELF leaves out where they are the source (own[i] == jj).
+template <bool SELF, bool SHARED>
+__device__ __forceinline__ void direct_run(const float4 *__restrict__ S, const float4 *__restrict__ pos, int tile,
+                                           int j, int count, const DirectNodes &r, unsigned base,
+                                           unsigned top, const int (&own)[kDirOwn], float2 (&acc)[kDirOwn][2])
+{
+    const float2 minus = dup(-1.0f);
+#pragma unroll 2
+    for (int u = 0; u < count; ++u) {
+        const int jj = j + u;
+        const float4 q = pos[jj];
+        float inv[kDirOwn], tau[kDirOwn];
+        float2 line = dup(0.0f);   // SHARED: the four lie on one row
+        if constexpr (SHARED) {
+            const float dy = r.y[0].x + q.y, dz = r.z[0].x + q.z;
+            line = dup(fmaf(dy, dy, dz * dz));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 dx = __fadd2_rn(r.x[h], dup(q.x));
+            if constexpr (!SHARED) {
+                const float2 dy = __fadd2_rn(r.y[h], dup(q.y)), dz = __fadd2_rn(r.z[h], dup(q.z));
+                line = __ffma2_rn(dy, dy, __fmul2_rn(dz, dz));
+            }
+            const float2 R2 = __ffma2_rn(dx, dx, line);
+            const float2 v = make_float2(rsqrt_ftz(R2.x), rsqrt_ftz(R2.y));
+            const float2 t = __fmul2_rn(R2, v);   // distances are in light steps c dt: this is tau
+            inv[2 * h] = v.x; inv[2 * h + 1] = v.y;
+            tau[2 * h] = t.x; tau[2 * h + 1] = t.y;
+        }
+        if constexpr (SELF) {
+#pragma unroll
+            for (int i = 0; i < kDirOwn; ++i)
+                if (own[i] == jj) inv[i] = tau[i] = 0.0f;
+        }
+        if constexpr (SHARED) {
+            // the earliest of the four lag intervals and the one after it:
+            // x0 + min(u, 1) (x1 - x0) + max(u - 1, 0) (x2 - x1), u = tau - m
+            const float t = __fadd_rd(fminf(fminf(tau[0], tau[1]), fminf(tau[2], tau[3])), kFloorShift);
+            const float m0 = t - kFloorShift, m1 = m0 + 1.0f;
+            const float4 *s = S + min(__float_as_uint(t) - base, top) * (unsigned)(tile + 1) + jj;
+            const float4 x0 = s[0], x1 = s[tile + 1], x2 = s[2 * (tile + 1)];
+            const float2 da = __ffma2_rn(lo2(x0), minus, lo2(x1)), db = __ffma2_rn(hi2(x0), minus, hi2(x1));
+            const float2 ea = __ffma2_rn(lo2(x1), minus, lo2(x2)), eb = __ffma2_rn(hi2(x1), minus, hi2(x2));
+#pragma unroll
+            for (int i = 0; i < kDirOwn; ++i) {
+                const float2 w = dup(__saturatef(tau[i] - m0)), e = dup(__saturatef(tau[i] - m1));
+                acc[i][0] = __ffma2_rn(dup(inv[i]), __ffma2_rn(e, ea, __ffma2_rn(w, da, lo2(x0))), acc[i][0]);
+                acc[i][1] = __ffma2_rn(dup(inv[i]), __ffma2_rn(e, eb, __ffma2_rn(w, db, hi2(x0))), acc[i][1]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kDirOwn; ++i) {
+                const float t = __fadd_rd(tau[i], kFloorShift);
+                const float2 w = dup(tau[i] - (t - kFloorShift));
+                const float4 *s = S + min(__float_as_uint(t) - base, top) * (unsigned)(tile + 1) + jj;
+                const float4 x0 = s[0], x1 = s[tile + 1];
+                const float2 da = __ffma2_rn(lo2(x0), minus, lo2(x1)), db = __ffma2_rn(hi2(x0), minus, hi2(x1));
+                acc[i][0] = __ffma2_rn(dup(inv[i]), __ffma2_rn(w, da, lo2(x0)), acc[i][0]);
+                acc[i][1] = __ffma2_rn(dup(inv[i]), __ffma2_rn(w, db, hi2(x0)), acc[i][1]);
+            }
+        }
+    }
+}
+
+// The target node at place i (0 .. 127) of block b of target T, or -1: groups
+// of four along a row, the last of a row padded (T.groups per row), or
+// consecutive nodes (T.groups = 0).
+__device__ __forceinline__ long long direct_node(const DirectTarget &T, int b, int i)
+{
+    const long long p = (long long)(b - T.block0) * kDirTargets + i;
+    if (T.groups == 0) return p < T.n ? p : -1;
+    const long long g = p / kDirOwn, line = g / T.groups;
+    const int x = (int)(g - line * T.groups) * kDirOwn + (i & (kDirOwn - 1));
+    return x < T.nx && line < (long long)T.ny * T.nz ? line * T.nx + x : -1;
+}
+
+// blockIdx.x: 128 target places (DirectTarget::block0), blockIdx.y: part of
+// the sources.  part: [target's part0 + split * 4 n + f n + k] when gridDim.y > 1.
+__global__ void __launch_bounds__(kDirThreads, 2)
+    k_direct(const DirectTarget *__restrict__ tgts, int ntgt, const DirectPair *__restrict__ pairs, OutPtrs out,
+             float *__restrict__ part, int tile, int max_nlag, long long step, int clamp, double inv_cdt, float inv_c)
 {
     extern __shared__ float4 smem_f4[];
-    float *sm = reinterpret_cast<float *>(smem_f4);
-    const int b = blockIdx.x;
+    float4 *S = smem_f4;   // two buffers of samples [nlag + 3][tile + 1] and positions [tile] (-x, -y, -z)
+    const int rows_max = max_nlag + 3, buf_elems = direct_buf_elems(max_nlag, tile);
+    float4 *sums = S + 2 * buf_elems;                                          // [warp][own][sum, comp][lane]
+    long long *row = reinterpret_cast<long long *>(sums + kDirSums);           // [nlag + 3]: slot offsets
+    const int b = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
     int lo = 0, hi = ntgt;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (tgts[mid].block0 <= b) lo = mid; else hi = mid;
     }
-    const DirectTarget T = tgts[lo];
+    const DirectTarget &T = tgts[lo];
     if (step < 0) step = *T.d_step;   // graph replay: the step from the device counter
-    const long long k = (long long)(b - T.block0) * kDirThreads + threadIdx.x;
-    const bool valid = k < T.n;
-    const int ix = (int)(k % T.nx), iy = (int)((k / T.nx) % T.ny), iz = (int)(k / ((long long)T.nx * T.ny));
-
-    float sum[4] = {0.f, 0.f, 0.f, 0.f}, comp[4] = {0.f, 0.f, 0.f, 0.f};
-
-    float *sx = sm, *sy = sx + kDirTile, *sz = sy + kDirTile;
-    float *S = sz + kDirTile;   // [nlag][4][kDirTile]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int share = tile / kDirWarps;   // sources of a warp in a full tile
+    float4 *mine = sums + warp * (kDirSums / kDirWarps) + lane;   // this thread's: + 64 i, + 64 i + 32
+#pragma unroll
+    for (int i = 0; i < 2 * kDirOwn; ++i) mine[32 * i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 
     for (int p = T.p0; p < T.p1; ++p) {
-        const DirectPair P = pairs[p];
-        // target node relative to the source origin, once in FP64
-        const float rx = (float)(P.dx + T.ht * ix), ry = (float)(P.dy + T.ht * iy),
-                    rz = (float)(P.dz + T.ht * iz);
-        for (long long j0 = 0; j0 < P.n_s; j0 += kDirTile) {
-            const int cnt = (int)min((long long)kDirTile, P.n_s - j0);
-            __syncthreads();
-            for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+        const DirectPair &P = pairs[p];
+        const int rows = P.nlag + 3;
+        DirectNodes r;   // once in FP64
+        {
+            float v[3][kDirOwn];
+            long long first = 0;
+#pragma unroll
+            for (int i = 0; i < kDirOwn; ++i) {   // a place without a node repeats the thread's first (or the last of all)
+                long long node = direct_node(T, b, lane * kDirOwn + i);
+                if (node < 0) node = i > 0 ? first : T.n - 1;
+                if (i == 0) first = node;
+                const long long line = node / T.nx;
+                v[0][i] = (float)((P.dx + T.ht * (int)(node - line * T.nx)) * inv_cdt);
+                v[1][i] = (float)((P.dy + T.ht * (int)(line % T.ny)) * inv_cdt);
+                v[2][i] = (float)((P.dz + T.ht * (int)(line / T.ny)) * inv_cdt);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                r.x[h] = make_float2(v[0][2 * h], v[0][2 * h + 1]);
+                r.y[h] = make_float2(v[1][2 * h], v[1][2 * h + 1]);
+                r.z[h] = make_float2(v[2][2 * h], v[2][2 * h + 1]);
+            }
+        }
+        // low bits of floor(tau) + 2^23, less the lag of sample row 0
+        const unsigned base = __float_as_uint(kFloorShift) + (unsigned)(P.lag_lo - 1), top = (unsigned)P.nlag;
+        __syncthreads();   // the rows of the pair before are read
+        for (int i = threadIdx.x; i < rows; i += kDirThreads) {
+            long long j = step - (P.lag_lo + max(0, min(i - 1, P.nlag - 1)));
+            if (clamp && j < 0) j = 0;
+            row[i] = (j % P.depth) * 4 * P.n_s;
+        }
+        // sources j0 .. of a tile into buffer `buf`: positions, and the samples
+        // by asynchronous copies (a tile ahead of the sums)
+        const float hs = (float)(P.hs * inv_cdt);
+        const long long j_end = P.n_s * (split + 1) / nsplit;
+        const auto stage = [&](long long j0, int buf) {
+            const int cnt = (int)min((long long)tile, j_end - j0);
+            float4 *Sb = S + buf * buf_elems, *pb = Sb + rows_max * (tile + 1);
+            for (int i = threadIdx.x; i < cnt; i += kDirThreads) {
                 const long long q = j0 + i;
-                sx[i] = P.hs * (float)(q % P.nx_s);
-                sy[i] = P.hs * (float)((q / P.nx_s) % P.ny_s);
-                sz[i] = P.hs * (float)(q / ((long long)P.nx_s * P.ny_s));
-            }
-            for (int i = threadIdx.x; i < P.nlag * 4 * kDirTile; i += blockDim.x) {
-                const int jj = i % kDirTile, fl = i / kDirTile;
-                const int f = fl & 3, li = fl >> 2;
-                float v = 0.0f;
-                if (jj < cnt) {
-                    long long j = step - (P.lag_lo + li);
-                    if (clamp && j < 0) j = 0;
-                    v = P.raw[((j % P.depth) * 4 + f) * P.n_s + j0 + jj];
+                int x, y, z;
+                if (q < 0x7fffffffLL) {
+                    const unsigned q32 = (unsigned)q, l = q32 / (unsigned)P.nx_s;
+                    x = (int)(q32 - l * (unsigned)P.nx_s);
+                    z = (int)(l / (unsigned)P.ny_s);
+                    y = (int)l - z * P.ny_s;
+                } else {
+                    x = (int)(q % P.nx_s); y = (int)((q / P.nx_s) % P.ny_s); z = (int)(q / ((long long)P.nx_s * P.ny_s));
                 }
-                S[i] = v;
+                pb[i] = make_float4(-hs * (float)x, -hs * (float)y, -hs * (float)z, 0.0f);
             }
-            __syncthreads();
-            if (!valid) continue;
-            for (int jj = 0; jj < cnt; ++jj) {
-                const float dx = rx - sx[jj], dy = ry - sy[jj], dz = rz - sz[jj];
-                const float R2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (P.is_self && j0 + jj == k) {
+            for (int i = threadIdx.x; i < rows * tile; i += kDirThreads) {
+                const int jj = i & (tile - 1), l = i / tile;
+                if (jj >= cnt) continue;
+                const float *src = P.raw + row[l] + j0 + jj;
+                float *dst = reinterpret_cast<float *>(Sb + l * (tile + 1) + jj);
 #pragma unroll
-                    for (int f = 0; f < 4; ++f) kahan_add(sum[f], comp[f], P.self_w * S[f * kDirTile + jj]);
-                    continue;
+                for (int f = 0; f < 4; ++f) cp_async4(dst + f, src + f * P.n_s);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        const long long j_first = P.n_s * split / nsplit;
+        __syncthreads();   // the rows' offsets
+        if (j_first < j_end) stage(j_first, 0);
+        int buf = 0;
+        for (long long j0 = j_first; j0 < j_end; j0 += tile, buf ^= 1) {
+            const int cnt = (int)min((long long)tile, j_end - j0);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();   // the tile is in, and the sums of the tile before are done with the other buffer
+            if (j0 + tile < j_end) stage(j0 + tile, buf ^ 1);
+            const float4 *Sb = S + buf * buf_elems, *pb = Sb + rows_max * (tile + 1);
+            int own[kDirOwn];   // the targets' places in this tile, if there (self pair)
+#pragma unroll
+            for (int i = 0; i < kDirOwn; ++i) {
+                own[i] = -1;
+                if (P.is_self) {
+                    const long long d = direct_node(T, b, lane * kDirOwn + i) - j0;
+                    if (d >= 0 && d < cnt) own[i] = (int)d;
                 }
-                const float inv = rsqrtf(R2);
-                const float tau = R2 * inv * inv_cdt;
-                const float m = floorf(tau);
-                const float w = tau - m;
-                int li = (int)m - P.lag_lo;
-                li = max(0, min(li, P.nlag - 2));
-                const float a = P.vol * inv;
-                const float *s0 = S + (li * 4) * kDirTile + jj;
-                const float *s1 = s0 + 4 * kDirTile;
+            }
+            const int end = min((warp + 1) * share, cnt);
+            for (int j = warp * share; j < end; j += kDirRun) {
+                const int count = min(kDirRun, end - j);
+                float2 acc[kDirOwn][2];
 #pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    const float x0 = s0[f * kDirTile], x1 = s1[f * kDirTile];
-                    kahan_add(sum[f], comp[f], a * fmaf(w, x1 - x0, x0));
+                for (int i = 0; i < kDirOwn; ++i) acc[i][0] = acc[i][1] = dup(0.0f);
+                if (P.is_self) {
+                    if (T.shared) direct_run<true, true>(Sb, pb, tile, j, count, r, base, top, own, acc);
+                    else direct_run<true, false>(Sb, pb, tile, j, count, r, base, top, own, acc);
+                } else {
+                    if (T.shared) direct_run<false, true>(Sb, pb, tile, j, count, r, base, top, own, acc);
+                    else direct_run<false, false>(Sb, pb, tile, j, count, r, base, top, own, acc);
+                }
+                const float2 vol = dup((float)(P.vol * inv_cdt));   // the run summed S / tau
+#pragma unroll
+                for (int i = 0; i < kDirOwn; ++i) {
+                    float4 sum = mine[64 * i], comp = mine[64 * i + 32];
+                    direct_add(sum, comp, __fmul2_rn(vol, acc[i][0]), __fmul2_rn(vol, acc[i][1]));
+                    if (own[i] >= j && own[i] < j + count) {   // weight C h^2 at lag 0 (sample row 1)
+                        const float4 x = Sb[tile + 1 + own[i]];
+                        const float2 w = dup(P.self_w);
+                        direct_add(sum, comp, __fmul2_rn(w, lo2(x)), __fmul2_rn(w, hi2(x)));
+                    }
+                    mine[64 * i] = sum;
+                    mine[64 * i + 32] = comp;
                 }
             }
         }
     }
-    if (!valid) return;
-    const long long N = T.n;
+    // the eight warps' sums of each target, in warp order
+    __syncthreads();
+    for (int c = threadIdx.x; c < 4 * kDirTargets; c += kDirThreads) {
+        const int f = c / kDirTargets, i = c % kDirTargets;
+        const long long k = direct_node(T, b, i);
+        if (k < 0) continue;
+        float s = 0.0f, e = 0.0f;
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        float *o = f == 0 ? out.phi[T.dom] + k : out.A[T.dom] + (long long)(f - 1) * N + k;
-        float v = sum[f] - comp[f];
+        for (int wv = 0; wv < kDirWarps; ++wv) {
+            const float *v4 = reinterpret_cast<const float *>(
+                sums + wv * (kDirSums / kDirWarps) + 64 * (i % kDirOwn) + i / kDirOwn);
+            kahan_add(s, e, v4[f] - v4[32 * 4 + f]);
+        }
+        float v = s - e;
+        if (nsplit > 1) {
+            part[T.part0 + ((long long)split * 4 + f) * T.n + k] = v;
+            continue;
+        }
+        float *o = f == 0 ? out.phi[T.dom] + k : out.A[T.dom] + (long long)(f - 1) * T.n + k;
         if (f > 0) v *= inv_c;
         if (T.accumulate) v += *o;
         *o = v;
     }
 }
 
+// The parts of each target in order (blocks as k_direct's; 16 B per node and
+// part, a few percent of the sums' time).
+__global__ void __launch_bounds__(kDirThreads)
+    k_direct_sum(const DirectTarget *__restrict__ tgts, int ntgt, OutPtrs out, const float *__restrict__ part,
+                 int nsplit, float inv_c)
+{
+    const int b = blockIdx.x;
+    int lo = 0, hi = ntgt;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (tgts[mid].block0 <= b) lo = mid; else hi = mid;
+    }
+    const DirectTarget &T = tgts[lo];
+    for (int c = threadIdx.x; c < 4 * kDirTargets; c += kDirThreads) {
+        const int f = c / kDirTargets;
+        const long long k = direct_node(T, b, c % kDirTargets);
+        if (k < 0) continue;
+        float s = 0.0f, e = 0.0f;
+        for (int i = 0; i < nsplit; ++i) kahan_add(s, e, part[T.part0 + ((long long)i * 4 + f) * T.n + k]);
+        float v = s - e;
+        float *o = f == 0 ? out.phi[T.dom] + k : out.A[T.dom] + (long long)(f - 1) * T.n + k;
+        if (f > 0) v *= inv_c;
+        if (T.accumulate) v += *o;
+        *o = v;
+    }
+}
+
+size_t direct_smem(int nlag, int tile)
+{
+    return 16 * (2 * (size_t)direct_buf_elems(nlag, tile) + kDirSums) + 8 * (size_t)(nlag + 3);
+}
+
+// The largest tile of which three blocks fit an SM (larger tiles stage more
+// per barrier); for the longest lag windows, one that fits at all.
+int direct_tile_of(int nlag)
+{
+    for (int tile : {128, 64})
+        if (direct_smem(nlag, tile) <= 72 * 1024) return tile;
+    return direct_smem(nlag, 32) <= 200 * 1024 ? 32 : 16;
+}
+
 }  // namespace
 
-size_t smem_direct(int max_nlag) { return sizeof(float) * (size_t)kDirTile * (3 + 4 * (size_t)max_nlag); }
+// Groups of four nodes per row of nx nodes, or 0 for consecutive nodes: four
+// along x share samples if light crosses them (3 h) within a step, and the
+// padding of the rows stays under a third of the places.
+int direct_groups(int nx, double h, double cdt, bool *shared)
+{
+    const int g = (nx + kDirOwn - 1) / kDirOwn;
+    *shared = 3.0 * h <= 0.999 * cdt && 2 * g * kDirOwn <= 3 * nx;
+    return *shared ? g : 0;
+}
 
-int direct_blocks(long long n) { return (int)((n + kDirThreads - 1) / kDirThreads); }
+int direct_blocks(const int n[3], int groups)
+{
+    const long long places = groups ? (long long)groups * kDirOwn * n[1] * n[2] : (long long)n[0] * n[1] * n[2];
+    return (int)((places + kDirTargets - 1) / kDirTargets);
+}
+
+// Parts of the sources: enough blocks for sixteen per SM, so that blocks of
+// unequal length leave no long tail, each with at least 512 sources.
+int direct_splits(int blocks, long long min_sources)
+{
+    const long long want = (16 * 152 + blocks - 1) / (blocks > 0 ? blocks : 1), most = min_sources / 512;
+    const long long s = want < most ? want : most;
+    return (int)(s < 1 ? 1 : s > 64 ? 64 : s);
+}
 
 cudaError_t open_direct_smem_limit(int max_optin)
 {
@@ -126,11 +403,15 @@ cudaError_t open_direct_smem_limit(int max_optin)
 }
 
 cudaError_t launch_direct(const DirectTarget *d_tgts, int ntgt, const DirectPair *d_pairs, const OutPtrs &out,
-                          int nblocks, size_t smem, long long step, int clamp, float inv_cdt, float inv_c,
-                          cudaStream_t s)
+                          float *part, int nsplit, int nblocks, int max_nlag, long long step, int clamp,
+                          double inv_cdt, float inv_c, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
-    k_direct<<<nblocks, kDirThreads, smem, s>>>(d_tgts, ntgt, d_pairs, out, step, clamp, inv_cdt, inv_c);
+    k_direct<<<dim3(nblocks, nsplit), kDirThreads, direct_smem(max_nlag, direct_tile_of(max_nlag)), s>>>(
+        d_tgts, ntgt, d_pairs, out, part, direct_tile_of(max_nlag), max_nlag, step, clamp, inv_cdt, inv_c);
+    cudaError_t e = cudaGetLastError();
+    if (e || nsplit == 1) return e;
+    k_direct_sum<<<nblocks, kDirThreads, 0, s>>>(d_tgts, ntgt, out, part, nsplit, inv_c);
     return cudaGetLastError();
 }
 

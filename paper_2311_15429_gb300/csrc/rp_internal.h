@@ -92,7 +92,7 @@ struct DirectPair {
     int nx_s, ny_s, nz_s;
     long long n_s;
     double dx, dy, dz;       // o_t - o_s
-    float hs;
+    double hs;
     float vol;               // hs^3
     float self_w;            // C hs^2 (self pair only)
     int is_self;
@@ -111,6 +111,8 @@ struct DirectTarget {
     int p0, p1;              // DirectPair range
     int block0;              // first block in the direct grid
     int accumulate;          // add onto the output (FFT pairs wrote it) instead of writing
+    int groups, shared;      // groups of four nodes per row (0: consecutive nodes); they share samples
+    long long part0;         // its parts' first float in the workspace ([split][4][n])
     const long long *d_step; // the step, for launches made with step < 0 (graph replay)
 };
 
@@ -261,9 +263,15 @@ cudaError_t launch_mac_inv_column(int size_class, bool comp, const InvTarget *d_
 cudaError_t launch_inv_plane(int size_class, bool tile, const InvTarget *d_tgts, int t0, int t1, int block_lo,
                              const OutPtrs &out, int nblocks, size_t smem, float inv_c, long long step,
                              cudaStream_t s);
+// part: the workspace of nsplit parts of the sources per target (unused for one)
 cudaError_t launch_direct(const DirectTarget *d_tgts, int ntgt, const DirectPair *d_pairs,
-                          const OutPtrs &out, int nblocks, size_t smem, long long step, int clamp,
-                          float inv_cdt, float inv_c, cudaStream_t s);
+                          const OutPtrs &out, float *part, int nsplit, int nblocks, int max_nlag, long long step,
+                          int clamp, double inv_cdt, float inv_c, cudaStream_t s);
+int direct_groups(int nx, double h, double cdt, bool *shared);
+int direct_blocks(const int n[3], int groups);
+int direct_splits(int blocks, long long min_sources);
+cudaError_t open_direct_smem_limit(int max_optin);
+constexpr int kDirMaxLags = 226;   // longest lag window of a direct pair
 
 // Ground-state split and graph-replay step counter (rp_ground.cu).
 cudaError_t launch_step_advance(long long *d_step, cudaStream_t s);
