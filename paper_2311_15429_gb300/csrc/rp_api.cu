@@ -137,22 +137,21 @@ rp_status build_twiddles(rp_ctx *ctx, std::map<int, const float2 *> &tw)
 namespace {
 
 
-// Pipeline depth of the bulk-copy-fed MAC for every cubic class of the plan;
-// the register-blocked MAC serves the plan if some class cannot hold two
-// field stages.
+// The fields of a block's unit and the pipeline depth of the bulk-copy-fed MAC
+// for every launch of the plan; the general MAC serves the plan if some launch
+// cannot hold two field stages.
 rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
 {
     ctx->tma = false;
-    for (int cls : {32, 48, 64, 96, 128, 192}) {
-        int n = mac_tma_stages(cls, max_optin, ctx->comp);
-        if (ctx->cfg.mac_stages >= 2) n = std::min(n, ctx->cfg.mac_stages);
-        ctx->mac_stages[class_slot(cls)] = n;
-        if (n < 2) {
-            for (const InvTarget &I : ctx->inv)
-                if (size_class(I.ax, I.ay, I.az) == cls) {
-                    ctx->last_error = "bulk-copy pipeline too shallow: register-blocked MAC in use";
-                    return RP_OK;
-                }
+    for (LaunchGroup &g : ctx->inv_groups) {
+        const int cls = column_class(g.cls);
+        if (cls == 0) continue;
+        g.fields = mac_tma_fields(cls, ctx->comp, g.blk1 - g.blk0, ctx->sm_count);
+        g.stages = mac_tma_stages(cls, max_optin, g.fields);
+        if (ctx->cfg.mac_stages >= 2) g.stages = std::min(g.stages, ctx->cfg.mac_stages);
+        if (g.stages < 2) {
+            ctx->last_error = "bulk-copy pipeline too shallow: general MAC in use";
+            return RP_OK;
         }
     }
     ctx->tma = true;
@@ -736,14 +735,14 @@ rp_status autotune_mac(rp_ctx *ctx)
     rp_status st = RP_OK;
     const long long step = ctx->max_lag;   // every (step - lag) is a valid slot
     for (const LaunchGroup &g : ctx->inv_groups) {
-        if (g.cls <= 0 || st) continue;
-        const int slot = class_slot(g.cls), ntiles = g.blk1 - g.blk0;
+        const int cls = column_class(g.cls);
+        if (cls == 0 || st) continue;
+        const int slot = class_slot(cls), ntiles = g.blk1 - g.blk0;
         float best = 1e30f;
         for (int cw : {8, 12, 16}) {
             auto go = [&] {
-                return launch_mac_tma(g.cls, cw, false, ctx->d_inv, g.i0, g.i1, g.blk0, ntiles, ctx->d_entries, step, 0,
-                                      ctx->mac_stages[slot], std::min(ntiles, ctx->sm_count), ctx->d_err,
-                                      ctx->stream);
+                return launch_mac_tma(cls, cw, false, ctx->d_inv, g.i0, g.i1, g.blk0, ntiles, ctx->d_entries, step, 0,
+                                      g.fields, g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
             };
             cudaError_t e = go();
             if (!e) e = cudaEventRecord(a, ctx->stream);
@@ -1012,9 +1011,10 @@ rp_status rp_finalize(rp_ctx *ctx)
     std::map<int, const float2 *> tw;
     {   // the plane passes' form per class, from its forward plane blocks
         int blocks[7] = {};
-        for (size_t r = 0; r < ring_keys.size(); ++r) blocks[class_slot(ring_class((int)r))] += 4 * ctx->doms[ring_keys[r].first].n[2];
+        for (size_t r = 0; r < ring_keys.size(); ++r)
+            blocks[class_slot(plane_class(ring_class((int)r)))] += 4 * ctx->doms[ring_keys[r].first].n[2];
         for (size_t r = 0; r < ring_keys.size(); ++r) {
-            const int cls = ring_class((int)r);
+            const int cls = plane_class(ring_class((int)r));
             ctx->fwd_tile[class_slot(cls)] = plane_tile_form(cls, blocks[class_slot(cls)], false);
         }
     }
@@ -1039,7 +1039,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         ctx->spectral_bytes += (long long)R.depth * R.slot_elems * (long long)sizeof(float2);
         ctx->spec_depth = std::max(ctx->spec_depth, R.depth);
         {
-            const int c = size_class(R.ax, R.ay, R.az), cs = class_slot(c);
+            const int c = plane_class(size_class(R.ax, R.ay, R.az)), cs = class_slot(c);
             const size_t need = smem_fwd_plane(c, ctx->fwd_tile[cs], R.ny, R.ax);
             ctx->smem_plane_cls[cs] = std::max(ctx->smem_plane_cls[cs], need);
             ctx->smem_plane = std::max(ctx->smem_plane, need);
@@ -1070,9 +1070,11 @@ rp_status rp_finalize(rp_ctx *ctx)
                      [&](int x, int y) { return tgt_class(x) < tgt_class(y); });
     {   // the inverse plane pass's form per class, from its blocks
         int blocks[7] = {};
-        for (int t : tgt_order) blocks[class_slot(tgt_class(t))] += 4 * ctx->doms[t].n[2];
-        for (int t : tgt_order) ctx->inv_tile[class_slot(tgt_class(t))] =
-                plane_tile_form(tgt_class(t), blocks[class_slot(tgt_class(t))], true);
+        for (int t : tgt_order) blocks[class_slot(plane_class(tgt_class(t)))] += 4 * ctx->doms[t].n[2];
+        for (int t : tgt_order) {
+            const int cls = plane_class(tgt_class(t));
+            ctx->inv_tile[class_slot(cls)] = plane_tile_form(cls, blocks[class_slot(cls)], true);
+        }
     }
     for (int t : tgt_order) {
         const DomainDesc &T = ctx->doms[t];
@@ -1115,7 +1117,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         ctx->invp_blocks += 4 * I.nz;
         ctx->smem_mac = std::max(ctx->smem_mac, smem_mac_inv_column(I.az));
         {
-            const int c = size_class(I.ax, I.ay, I.az), cs = class_slot(c);
+            const int c = plane_class(size_class(I.ax, I.ay, I.az)), cs = class_slot(c);
             const size_t need = smem_inv_plane(c, ctx->inv_tile[cs], I.nx, I.ny, I.ax, I.ay);
             ctx->smem_inv_cls[cs] = std::max(ctx->smem_inv_cls[cs], need);
             ctx->smem_inv = std::max(ctx->smem_inv, need);
@@ -1370,11 +1372,11 @@ rp_status rp_finalize(rp_ctx *ctx)
         }
     }
 
-    // ---- bulk-copy MAC pipeline for the cubic classes
+    // ---- bulk-copy MAC pipeline
+    RP_CUDA(ctx, cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device));
     if ((st = plan_mac_tma(ctx, max_optin))) return st;
 
     // ---- far pairs
-    RP_CUDA(ctx, cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device));
     if (!(ctx->cfg.flags & RP_FLAG_DEFER_FAR) && (st = build_far(ctx, max_optin))) return st;
 
     // ---- device tables and kernel limits
@@ -1509,16 +1511,17 @@ rp_status enqueue_push(rp_ctx *ctx, int d0, int d1, const IoPtrs &in)
         }
     }
     for (const LaunchGroup &g : launches) {
+        const int cls = plane_class(g.cls);
         if ((st = timed_launch(ctx, RP_K_FWD_PLANE, "forward plane pass", [&] {
-                 return launch_fwd_plane(g.cls, ctx->fwd_tile[class_slot(g.cls)], rings, fin, g.i0, g.i1, g.blk0,
-                                         g.blk1 - g.blk0, ctx->smem_plane_cls[class_slot(g.cls)],
+                 return launch_fwd_plane(cls, ctx->fwd_tile[class_slot(cls)], rings, fin, g.i0, g.i1, g.blk0,
+                                         g.blk1 - g.blk0, ctx->smem_plane_cls[class_slot(cls)],
                                          (int)(step % std::max(1, ctx->cfg.far_batch)), ctx->stream);
              })))
             return st;
     }
     for (const LaunchGroup &g : launches) {
         if ((st = timed_launch(ctx, RP_K_FWD_COLUMN, "forward column pass", [&] {
-                 return launch_fwd_column(g.cls, rings, g.i0, g.i1, g.blk2_0, g.blk2_1 - g.blk2_0,
+                 return launch_fwd_column(column_class(g.cls), rings, g.i0, g.i1, g.blk2_0, g.blk2_1 - g.blk2_0,
                                           ctx->smem_col, kstep, ctx->stream);
              })))
             return st;
@@ -1914,13 +1917,11 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
     for (const LaunchGroup &g : ctx->inv_groups) {
         const int ntiles = g.blk1 - g.blk0;
         if ((st = timed_launch(ctx, RP_K_MAC_INV_COLUMN, "MAC + inverse column pass", [&] {
-                 if (ctx->tma && g.cls > 0)
-                     return launch_mac_tma(g.cls, ctx->mac_cw[class_slot(g.cls)], ctx->comp, ctx->d_inv, g.i0, g.i1,
-                                           g.blk0,
-                                           ntiles, ctx->d_entries, kstep, clamp,
-                                           ctx->mac_stages[class_slot(g.cls)],
-                                           std::min(ntiles, ctx->sm_count), ctx->d_err, ctx->stream);
-                 return launch_mac_inv_column(g.cls, ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0, ctx->d_entries, ntiles,
+                 if (const int cls = column_class(g.cls); ctx->tma && cls > 0)
+                     return launch_mac_tma(cls, ctx->mac_cw[class_slot(cls)], ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0,
+                                           ntiles, ctx->d_entries, kstep, clamp, g.fields, g.stages, ctx->sm_count,
+                                           ctx->d_err, ctx->stream);
+                 return launch_mac_inv_column(ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0, ctx->d_entries, ntiles,
                                               ctx->smem_mac, kstep, clamp, ctx->stream);
              })))
             return st;
@@ -1943,9 +1944,10 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
             return st;
     }
     for (const LaunchGroup &g : ctx->inv_groups) {
+        const int cls = plane_class(g.cls);
         if ((st = timed_launch(ctx, RP_K_INV_PLANE, "inverse plane pass", [&] {
-                 return launch_inv_plane(g.cls, ctx->inv_tile[class_slot(g.cls)], ctx->d_inv, g.i0, g.i1, g.blk2_0,
-                                         out, g.blk2_1 - g.blk2_0, ctx->smem_inv_cls[class_slot(g.cls)], inv_c, kstep,
+                 return launch_inv_plane(cls, ctx->inv_tile[class_slot(cls)], ctx->d_inv, g.i0, g.i1, g.blk2_0,
+                                         out, g.blk2_1 - g.blk2_0, ctx->smem_inv_cls[class_slot(cls)], inv_c, kstep,
                                          ctx->stream);
              })))
             return st;
@@ -2510,7 +2512,7 @@ rp_status rp_query(rp_ctx *ctx, rp_stats *out)
     for (const PairPlan &p : ctx->pairs) out->npairs_other += p.kind == RP_PAIR_OTHER;
     out->mac_warps = 0;
     for (const LaunchGroup &g : ctx->inv_groups)
-        if (g.cls > 0 && ctx->tma) out->mac_warps = ctx->mac_cw[class_slot(g.cls)];
+        if (column_class(g.cls) > 0 && ctx->tma) out->mac_warps = ctx->mac_cw[class_slot(column_class(g.cls))];
     out->npairs_direct = 0;
     out->npairs_fft = 0;
     for (const PairPlan &p : ctx->pairs) {

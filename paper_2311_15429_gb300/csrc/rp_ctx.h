@@ -43,7 +43,7 @@ struct ProfRec {
 // One launch of a kernel pair over a contiguous range [i0, i1) of rings (or
 // targets) of one size class: first kernel's blocks [blk0, blk1), second
 // kernel's blocks [blk2_0, blk2_1).
-// Index of a kernel size class (0: the run-time shape) in the per-class tables.
+// Index of a kernel's compiled length (0: the run-time shape) in the per-class tables.
 inline int class_slot(int cls)
 {
     switch (cls) {
@@ -53,10 +53,11 @@ inline int class_slot(int cls)
 }
 
 struct LaunchGroup {
-    int cls;
+    int cls;                 // size_class: plane passes' and column passes' kernels
     int i0, i1;
     int blk0, blk1;
     int blk2_0, blk2_1;
+    int fields = 0, stages = 0;   // MAC launches: fields of a block's unit, field stages of its pipeline
 };
 
 // History spill (RP_FLAG_HISTORY_SPILL).  A source domain with a spilled
@@ -178,7 +179,6 @@ struct rp_ctx {
     DirectPair *d_dpairs = nullptr;
     RawRing *d_raw = nullptr;
     bool tma = false;                // TMA-fed MAC available for the cubic classes
-    int mac_stages[7] = {};          // pipeline depth per class (index by class_slot)
     int mac_cw[7] = {16, 16, 16, 16, 16, 16, 16};   // consumer warps of the MAC per class
     int sm_count = 0;
     int *d_err = nullptr;            // set by a kernel whose bounded wait ran out

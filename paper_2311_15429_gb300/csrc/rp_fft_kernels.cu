@@ -18,9 +18,9 @@
 // k_inv_plane16 run the two-stage shared-memory tile transform of rp_fft.cuh
 // (M = 16 B: the plane passes for M = 64, 96, 128, the column pass also for
 // 192).  k_fwd_plane, k_fwd_column and k_inv_plane run the lane-shuffle line
-// transform for the other cubic sizes (32, 48, and 192 for the plane passes)
-// and for M = 0 (any supported shape, read at run time).  The MAC with its
-// inverse column transform is instantiated for every class.
+// transform for the other sizes (32, 48, and 192 for the plane passes) and for
+// M = 0 (any supported shape, read at run time).  The MAC here serves shapes
+// with no column class.
 #include <cuda_runtime.h>
 
 #include "rp_fft.cuh"
@@ -310,8 +310,8 @@ __global__ void __launch_bounds__(kColumnThreads) k_fwd_column(const FwdRing *__
     const int r = owner_of(rings, r0, r1, b, &FwdRing::tile0);
     const FwdRing &R = rings[r];
     const Axis az = axis_of<M>(R.az);
-    const int my = M ? M : R.ay.M, mz = az.M, nz = R.nz;
-    const int kx = M ? M / 2 + 1 : R.kx;
+    const int my = R.ay.M, mz = az.M, nz = R.nz;   // M > 0: mz = M, my a multiple of 16
+    const int kx = R.kx;
     const int ntile = (my + kTileY - 1) / kTileY;
     const int local = b - R.tile0;
     const int kxi = local / ntile, ky0 = (local % ntile) * kTileY;
@@ -387,14 +387,14 @@ template <int M>
 __global__ void __launch_bounds__(kColumn16Threads) k_fwd_column16(const FwdRing *__restrict__ rings, int r0, int r1,
                                                                     int block_lo, long long step)
 {
-    constexpr int B = M / 16, kx = M / 2 + 1, ntile = M / kTileY;
+    constexpr int B = M / 16;
     static_assert(tile16_class(M), "k_fwd_column16: M = 16 B, B even");
     extern __shared__ float4 smem_f4[];
     float2 *sm = reinterpret_cast<float2 *>(smem_f4);
     const int b = blockIdx.x + block_lo;
     const int r = owner_of(rings, r0, r1, b, &FwdRing::tile0);
     const FwdRing &R = rings[r];
-    const int nz = R.nz;
+    const int nz = R.nz, my = R.ay.M, kx = R.kx, ntile = my / kTileY;
     const int local = b - R.tile0;
     const int kxi = local / ntile, kyt = local % ntile;
     float2 *tw = sm;
@@ -411,9 +411,9 @@ __global__ void __launch_bounds__(kColumn16Threads) k_fwd_column16(const FwdRing
     const int t64 = threadIdx.x & 63, p = t64 & 7, zr = t64 >> 3;   // column pair p, rows zr + 8 j
     float2 *Vf = V + f * M * kTileY;
     {
-        const long long t1_field = (long long)kx * nz * M;
-        const float2 *src = R.t1 + f * t1_field + (long long)kxi * nz * M + kyt * kTileY + 2 * p;
-        for (int z = zr; z < nz; z += 8) cp_async16(Vf + z * kTileY + 2 * p, src + (long long)z * M);
+        const long long t1_field = (long long)kx * nz * my;
+        const float2 *src = R.t1 + f * t1_field + (long long)kxi * nz * my + kyt * kTileY + 2 * p;
+        for (int z = zr; z < nz; z += 8) cp_async16(Vf + z * kTileY + 2 * p, src + (long long)z * my);
         cp_async_wait_all();
     }
     asm volatile("bar.sync %0, 64;" ::"r"(1 + f) : "memory");
@@ -439,10 +439,11 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float x)
 }
 
 // Spectral multiply-accumulate over the target's (source, lag) entries for
-// one (kx, 16-ky) column block and all four fields, then the inverse FFT
+// one (kx, 16-ky) column block and all four fields, any shape (the shapes with
+// no column class; the others run k_mac_tma), then the inverse FFT
 // along z of the 64 columns; rows z < nz of the target go to T2.  COMP: the
 // sum over entries is Kahan-compensated per spectral coefficient.
-template <int M, bool COMP>
+template <bool COMP>
 __global__ void __launch_bounds__(kThreads) k_mac_inv_column(const InvTarget *__restrict__ tgts, int t0, int t1,
                                                                int block_lo, const MacEntry *__restrict__ entries,
                                                                long long step, int clamp)
@@ -452,16 +453,15 @@ __global__ void __launch_bounds__(kThreads) k_mac_inv_column(const InvTarget *__
     const int b = blockIdx.x + block_lo;
     const int t = owner_of(tgts, t0, t1, b, &InvTarget::tile0);
     const InvTarget &T = tgts[t];
-    const Axis az = axis_of<M>(T.az);
-    const int my = M ? M : T.ay.M, mz = az.M;
-    const int kx = M ? M / 2 + 1 : T.kx;
+    const Axis az = T.az;
+    const int my = T.ay.M, mz = az.M;
+    const int kx = T.kx;
     const int ntile = (my + kTileY - 1) / kTileY;
     const int local = b - T.tile0;
     const int kxi = local / ntile, ky0 = (local % ntile) * kTileY;
     const int ncols = min(kTileY, my - ky0);
     const long long col0 = (long long)(kxi * ntile + ky0 / kTileY) * mz * kTileY;   // tile in a kernel spectrum
     const long long fstride = (long long)mz * kTileY;                             // field tile in a ring slot
-    const long long sbase = 3 * col0;   // + col0: the tile's first field tile in a ring slot (4 per tile)
     const int fs = mz * kTileYPad;
 
     float2 *tw = sm;
@@ -471,177 +471,52 @@ __global__ void __launch_bounds__(kThreads) k_mac_inv_column(const InvTarget *__
     pdl_wait();   // the newest ring slot is written by the column pass
     if (step < 0) step = *T.d_step;   // graph replay: the step from the device counter
 
-    if constexpr (M > 0) {
-        // Thread (p, r0) owns ky columns 2p, 2p+1 and kz rows r0 + 32 i.  All
-        // operands of an entry (kernel + four fields, CH rows) are loaded
-        // before the multiply-adds, so 5*CH 16-byte loads are in flight.
-        constexpr int ROWS = (M + 31) / 32;
-        constexpr int CH = ROWS < 3 ? ROWS : 3;
-        constexpr int NCH = (ROWS + CH - 1) / CH;
-        const int p = threadIdx.x & 7, r0 = threadIdx.x >> 3;
-#pragma unroll 1
-        for (int ch = 0; ch < NCH; ++ch) {
-            float4 a[4][CH], cmp[4][COMP ? CH : 1];
+    for (int i = threadIdx.x; i < 4 * fs; i += blockDim.x) acc[i] = make_float2(0.0f, 0.0f);
+    __syncthreads();
+    // Each thread owns the (kz, c) cells i = threadIdx.x + k*blockDim.x and
+    // sums every entry of one cell in registers (entries in order, the
+    // warp's lanes reading consecutive cells of an entry), then stores it.
+    for (int i = threadIdx.x; i < mz * kTileY; i += blockDim.x) {
+        const int kz = i / kTileY, c = i % kTileY;
+        if (c >= ncols) continue;
+        const long long off = kz * kTileY + c;
+        float2 v[4], cv[4];
 #pragma unroll
-            for (int f = 0; f < 4; ++f)
+        for (int f = 0; f < 4; ++f) v[f] = cv[f] = make_float2(0.0f, 0.0f);
+        for (int e = T.e0; e < T.e1; ++e) {
+            const MacEntry E = entries[e];
+            long long j = step - E.lag;
+            if (clamp && j < 0) j = 0;
+            const float2 *S = E.ring + (j % E.depth) * E.slot_elems + 4 * col0;
+            const float2 g = E.is_real ? make_float2(__ldg(static_cast<const float *>(E.g) + col0 + off), 0.0f)
+                                       : __ldg(static_cast<const float2 *>(E.g) + col0 + off);
 #pragma unroll
-                for (int j = 0; j < CH; ++j) a[f][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int f = 0; f < 4; ++f)
-#pragma unroll
-                for (int j = 0; j < (COMP ? CH : 1); ++j) cmp[f][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            long long off[CH];
-            bool ok[CH];
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const int row = r0 + 32 * (ch * CH + j);
-                ok[j] = row < M;
-                off[j] = col0 + (ok[j] ? row : 0) * kTileY + 2 * p;
-            }
-#pragma unroll 2
-            for (int e = T.e0; e < T.er; ++e) {   // self pair: real kernel
-                const MacEntry E = entries[e];
-                long long j = step - E.lag;
-                if (clamp && j < 0) j = 0;
-                const float2 *S = E.ring + (j % E.depth) * E.slot_elems + sbase;
-                const float *G = static_cast<const float *>(E.g);
-                float2 g[CH];
-                float4 s[4][CH];
-#pragma unroll
-                for (int jj = 0; jj < CH; ++jj) {
-                    g[jj] = __ldg(reinterpret_cast<const float2 *>(G + off[jj]));
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) s[f][jj] = ldg4(S + f * fstride + off[jj]);
-                }
-#pragma unroll
-                for (int jj = 0; jj < CH; ++jj)
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        if constexpr (COMP) {
-                            float4 &c = cmp[f][COMP ? jj : 0];
-                            kahan_add(a[f][jj].x, c.x, g[jj].x * s[f][jj].x);
-                            kahan_add(a[f][jj].y, c.y, g[jj].x * s[f][jj].y);
-                            kahan_add(a[f][jj].z, c.z, g[jj].y * s[f][jj].z);
-                            kahan_add(a[f][jj].w, c.w, g[jj].y * s[f][jj].w);
-                        } else {
-                            a[f][jj].x = fmaf(g[jj].x, s[f][jj].x, a[f][jj].x);
-                            a[f][jj].y = fmaf(g[jj].x, s[f][jj].y, a[f][jj].y);
-                            a[f][jj].z = fmaf(g[jj].y, s[f][jj].z, a[f][jj].z);
-                            a[f][jj].w = fmaf(g[jj].y, s[f][jj].w, a[f][jj].w);
-                        }
-                    }
-            }
-#pragma unroll 2
-            for (int e = T.er; e < T.e1; ++e) {   // other sources: complex kernel
-                const MacEntry E = entries[e];
-                long long j = step - E.lag;
-                if (clamp && j < 0) j = 0;
-                const float2 *S = E.ring + (j % E.depth) * E.slot_elems + sbase;
-                const float2 *G = static_cast<const float2 *>(E.g);
-                float4 g[CH];
-                float4 s[4][CH];
-#pragma unroll
-                for (int jj = 0; jj < CH; ++jj) {
-                    g[jj] = ldg4(G + off[jj]);
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) s[f][jj] = ldg4(S + f * fstride + off[jj]);
-                }
-#pragma unroll
-                for (int jj = 0; jj < CH; ++jj)
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        float4 &x = a[f][jj];
-                        const float4 gg = g[jj], ss = s[f][jj];
-                        if constexpr (COMP) {
-                            float4 &c = cmp[f][COMP ? jj : 0];
-                            kahan_add(x.x, c.x, fmaf(gg.x, ss.x, -gg.y * ss.y));
-                            kahan_add(x.y, c.y, fmaf(gg.x, ss.y, gg.y * ss.x));
-                            kahan_add(x.z, c.z, fmaf(gg.z, ss.z, -gg.w * ss.w));
-                            kahan_add(x.w, c.w, fmaf(gg.z, ss.w, gg.w * ss.z));
-                        } else {
-                            x.x = fmaf(gg.x, ss.x, fmaf(-gg.y, ss.y, x.x));
-                            x.y = fmaf(gg.x, ss.y, fmaf(gg.y, ss.x, x.y));
-                            x.z = fmaf(gg.z, ss.z, fmaf(-gg.w, ss.w, x.z));
-                            x.w = fmaf(gg.z, ss.w, fmaf(gg.w, ss.z, x.w));
-                        }
-                    }
-            }
-#pragma unroll
-            for (int jj = 0; jj < CH; ++jj) {
-                if (!ok[jj]) continue;
-                const int row = r0 + 32 * (ch * CH + jj);
-#pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    if constexpr (COMP) {
-                        const float4 &c = cmp[f][COMP ? jj : 0];
-                        a[f][jj] = make_float4(a[f][jj].x - c.x, a[f][jj].y - c.y, a[f][jj].z - c.z, a[f][jj].w - c.w);
-                    }
-                    float2 *d = acc + f * fs + row * kTileYPad + 2 * p;
-                    d[0] = make_float2(a[f][jj].x, a[f][jj].y);
-                    d[1] = make_float2(a[f][jj].z, a[f][jj].w);
+            for (int f = 0; f < 4; ++f) {
+                const float2 t = cmul(g, __ldg(S + f * fstride + off));
+                if constexpr (COMP) {
+                    kahan_add(v[f].x, cv[f].x, t.x);
+                    kahan_add(v[f].y, cv[f].y, t.y);
+                } else {
+                    v[f] = cadd(v[f], t);
                 }
             }
         }
-    } else {
-        for (int i = threadIdx.x; i < 4 * fs; i += blockDim.x) acc[i] = make_float2(0.0f, 0.0f);
-        __syncthreads();
-        // Each thread owns the (kz, c) cells i = threadIdx.x + k*blockDim.x and
-        // sums every entry of one cell in registers (entries in order, the
-        // warp's lanes reading consecutive cells of an entry), then stores it.
-        for (int i = threadIdx.x; i < mz * kTileY; i += blockDim.x) {
-            const int kz = i / kTileY, c = i % kTileY;
-            if (c >= ncols) continue;
-            const long long off = kz * kTileY + c;
-            float2 v[4], cv[4];
+        const int a_ = kz * kTileYPad + c;
 #pragma unroll
-            for (int f = 0; f < 4; ++f) v[f] = cv[f] = make_float2(0.0f, 0.0f);
-            for (int e = T.e0; e < T.e1; ++e) {
-                const MacEntry E = entries[e];
-                long long j = step - E.lag;
-                if (clamp && j < 0) j = 0;
-                const float2 *S = E.ring + (j % E.depth) * E.slot_elems + 4 * col0;
-                const float2 g = E.is_real ? make_float2(__ldg(static_cast<const float *>(E.g) + col0 + off), 0.0f)
-                                           : __ldg(static_cast<const float2 *>(E.g) + col0 + off);
-#pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    const float2 t = cmul(g, __ldg(S + f * fstride + off));
-                    if constexpr (COMP) {
-                        kahan_add(v[f].x, cv[f].x, t.x);
-                        kahan_add(v[f].y, cv[f].y, t.y);
-                    } else {
-                        v[f] = cadd(v[f], t);
-                    }
-                }
-            }
-            const int a_ = kz * kTileYPad + c;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) acc[f * fs + a_] = COMP ? make_float2(v[f].x - cv[f].x, v[f].y - cv[f].y) : v[f];
-        }
+        for (int f = 0; f < 4; ++f) acc[f * fs + a_] = COMP ? make_float2(v[f].x - cv[f].x, v[f].y - cv[f].y) : v[f];
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    LaneTw<lane_class(M), true> lt;
-    if constexpr (M > 0) lt.init(tw, lane & (az.L - 1));
-    ColumnFFT<M, true> cf{&lt, az, acc, fs, ncols, 4, T.nz, tw, lane, warp, nwarps};
-    run_radix<M>(az.R, cf);
+    ColumnFFT<0, true> cf{nullptr, az, acc, fs, ncols, 4, T.nz, tw, lane, warp, nwarps};
+    run_radix<0>(az.R, cf);
     __syncthreads();
     const int nz = T.nz;
     const long long t2_field = (long long)kx * nz * my;
     float2 *dst = T.t2 + (long long)kxi * nz * my + ky0;
-    if constexpr (M > 0) {
-        for (int i = threadIdx.x; i < 4 * nz * (kTileY / 2); i += blockDim.x) {
-            const int f = i / (nz * (kTileY / 2)), rem = i % (nz * (kTileY / 2));
-            const int zi = rem / (kTileY / 2), p = rem % (kTileY / 2);
-            const float2 *s = acc + f * fs + zi * kTileYPad + 2 * p;
-            *reinterpret_cast<float4 *>(dst + f * t2_field + (long long)zi * my + 2 * p) =
-                make_float4(s[0].x, s[0].y, s[1].x, s[1].y);
-        }
-    } else {
-        for (int i = threadIdx.x; i < 4 * nz * kTileY; i += blockDim.x) {
-            const int f = i / (nz * kTileY), rem = i % (nz * kTileY);
-            const int zi = rem / kTileY, c = rem % kTileY;
-            if (c < ncols) dst[f * t2_field + (long long)zi * my + c] = acc[f * fs + zi * kTileYPad + c];
-        }
+    for (int i = threadIdx.x; i < 4 * nz * kTileY; i += blockDim.x) {
+        const int f = i / (nz * kTileY), rem = i % (nz * kTileY);
+        const int zi = rem / kTileY, c = rem % kTileY;
+        if (c < ncols) dst[f * t2_field + (long long)zi * my + c] = acc[f * fs + zi * kTileYPad + c];
     }
 }
 
@@ -1210,11 +1085,14 @@ __global__ void __launch_bounds__(kPlaneBigThreads, 2) k_inv_plane_big(const Inv
 
 int size_class(const Axis &ax, const Axis &ay, const Axis &az)
 {
-    if (ax.M != ay.M || ax.M != az.M) return 0;
-    switch (ax.M) {
-    case 32: case 48: case 64: case 96: case 128: case 192: return ax.M;
-    default: return 0;
-    }
+    const auto compiled = [](int M) {
+        switch (M) {
+        case 32: case 48: case 64: case 96: case 128: case 192: return M;
+        default: return 0;
+        }
+    };
+    const int plane = ax.M == ay.M ? compiled(ax.M) : 0, column = ay.M % kTileY == 0 ? compiled(az.M) : 0;
+    return column << 8 | plane;
 }
 
 bool plane_tile_class(int size_class) { return plane16_class(size_class); }
@@ -1284,7 +1162,6 @@ static cudaError_t open_class_smem(int max_optin)
     } else {
         if ((e = open(k_fwd_column<M>))) return e;
     }
-    if ((e = open(k_mac_inv_column<M, false>)) || (e = open(k_mac_inv_column<M, true>))) return e;
     return cudaSuccess;
 }
 
@@ -1295,6 +1172,8 @@ cudaError_t open_kernel_smem_limits(int max_optin)
     if ((e = open_class_smem<M>(max_optin))) return e;
     RP_FOR_EACH_CLASS(RP_OPEN)
 #undef RP_OPEN
+    for (auto kern : {k_mac_inv_column<false>, k_mac_inv_column<true>})
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin))) return e;
     return cudaSuccess;
 }
 
@@ -1308,9 +1187,6 @@ cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, i
     k_ring_push<<<nblocks, kThreads, 0, s>>>(d_rings, in, pre, d0, d1, step);
     return cudaGetLastError();
 }
-
-#define RP_CASE(M, KERNEL, THREADS, ...) \
-    case M: if (cudaError_t e_ = launch_pdl(KERNEL<M>, dim3(nblocks), dim3(THREADS), smem, s, __VA_ARGS__)) return e_; break;
 
 template <int M>
 static cudaError_t launch_fwd_plane_cls(bool tile, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
@@ -1387,24 +1263,13 @@ cudaError_t launch_fwd_column(int cls, const FwdRing *d_rings, int r0, int r1, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_mac_inv_column(int cls, bool comp, const InvTarget *d_tgts, int t0, int t1, int block_lo,
+cudaError_t launch_mac_inv_column(bool comp, const InvTarget *d_tgts, int t0, int t1, int block_lo,
                                   const MacEntry *d_entries, int nblocks, size_t smem, long long step, int clamp,
                                   cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
-    switch (cls) {
-#define X(M)                                                                                                   \
-    case M:                                                                                                    \
-        if (cudaError_t e_ = launch_pdl(comp ? k_mac_inv_column<M, true> : k_mac_inv_column<M, false>,        \
-                                        dim3(nblocks), dim3(kThreads), smem, s, d_tgts, t0, t1, block_lo,      \
-                                        d_entries, step, clamp))                                               \
-            return e_;                                                                                         \
-        break;
-        RP_FOR_EACH_CLASS(X)
-#undef X
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return launch_pdl(comp ? k_mac_inv_column<true> : k_mac_inv_column<false>, dim3(nblocks), dim3(kThreads), smem, s,
+                      d_tgts, t0, t1, block_lo, d_entries, step, clamp);
 }
 
 cudaError_t launch_inv_plane(int cls, bool tile, const InvTarget *d_tgts, int t0, int t1, int block_lo,

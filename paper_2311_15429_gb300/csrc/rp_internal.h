@@ -227,12 +227,19 @@ struct OutPtrs {
 
 // ---- launchers (rp_fft_kernels.cu, rp_direct.cu) ----
 //
-// `size_class` selects the kernel instantiation: a cubic padded size M in
-// {32, 48, 64, 96, 128, 192} compiled with constant shapes, or 0 for the
-// general runtime-shaped kernels.  Rings [r0, r1) / targets [t0, t1) of one
-// launch share the class; `block_lo` is the first block of the range.
+// `size_class` selects the kernel instantiations of a padded shape, two in
+// one number: the plane passes' (M in {32, 48, 64, 96, 128, 192} where mx = my
+// = M) and the column passes' and the MAC's (mz in the same set where the ky
+// tiles are whole, my a multiple of 16), each 0 for the general
+// runtime-shaped kernels.  An elongated box so takes the kernels of its
+// length along z whatever its cross-section: 16 x 16 x 96 wires (padded 32 x
+// 32 x 192, 40 entries a target) 469 -> 68 us per step.  Rings [r0, r1)
+// / targets [t0, t1) of one launch share the class; `block_lo` is the first
+// block of the range.
 
 int size_class(const Axis &ax, const Axis &ay, const Axis &az);
+inline int plane_class(int size_class) { return size_class & 255; }
+inline int column_class(int size_class) { return size_class >> 8; }
 
 cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, int d1,
                              const int *h_block0, int nblocks, long long step,
@@ -257,7 +264,7 @@ cudaError_t launch_fwd_plane(int size_class, bool tile, const FwdRing *d_rings, 
                              int block_lo, int nblocks, size_t smem, int far_slot, cudaStream_t s);
 cudaError_t launch_fwd_column(int size_class, const FwdRing *d_rings, int r0, int r1, int block_lo,
                               int nblocks, size_t smem, long long step, cudaStream_t s);
-cudaError_t launch_mac_inv_column(int size_class, bool comp, const InvTarget *d_tgts, int t0, int t1, int block_lo,
+cudaError_t launch_mac_inv_column(bool comp, const InvTarget *d_tgts, int t0, int t1, int block_lo,
                                   const MacEntry *d_entries, int nblocks, size_t smem, long long step,
                                   int clamp, cudaStream_t s);
 cudaError_t launch_inv_plane(int size_class, bool tile, const InvTarget *d_tgts, int t0, int t1, int block_lo,
@@ -282,16 +289,17 @@ cudaError_t launch_ground_delta(const float *rho, const float *J, const float *g
 cudaError_t launch_fields(int nx, int ny, int nz, double h, double c, double dt, const float *phi, const float *A,
                           const float *A1, const float *A2, float *E, float *B, cudaStream_t s);
 
-// TMA-fed MAC (rp_mac_tma.cu): cubic classes 32..192 only.
-int mac_tma_stages(int M, int smem_optin, bool comp);
+// TMA-fed MAC (rp_mac_tma.cu): column classes 32..192.
+int mac_tma_fields(int M, bool comp, int ntiles, int sms);   // fields of a block's unit of work
+int mac_tma_stages(int M, int smem_optin, int fields);
 cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_t s);
-size_t mac_tma_smem(int M, int nstages, bool comp);
+size_t mac_tma_smem(int M, int nstages, int fields);
 cudaError_t open_mac_tma_smem_limit(int max_optin);
 // comp: the Kahan-compensated variant (consumer_warps must be kCompWarps)
 constexpr int kCompWarps = 12;
 cudaError_t launch_mac_tma(int cls, int consumer_warps, bool comp, const InvTarget *d_tgts, int t0, int t1,
-                           int tile_lo, int ntiles, const MacEntry *d_entries, long long step, int clamp, int nstages,
-                           int grid, int *d_err, cudaStream_t s);
+                           int tile_lo, int ntiles, const MacEntry *d_entries, long long step, int clamp, int fields,
+                           int nstages, int sms, int *d_err, cudaStream_t s);
 
 // tcgen05 bf16 GEMM (rp_gemm_tc.cu): D (M x N fp32) = A (M x K) * B (N x K)^T
 bool encode_bf16_rows(void *encode_fn, struct CUtensorMap_st *map, const void *base, uint64_t rows,

@@ -1,12 +1,13 @@
 // Spectral multiply-accumulate + inverse column FFT, fed by the tensor memory
 // accelerator.
 //
-// Same arithmetic as k_mac_inv_column (the sum over a target's (source, lag)
+// For every padded shape with a column class (rp_internal.h).  Same arithmetic as k_mac_inv_column (the sum over a target's (source, lag)
 // entries of G_m * S(l - m), Eq. 12 in the spectral domain, then the inverse
 // FFT along z kept to the target's z < nz), restructured so that the
 // operands stream through shared memory asynchronously:
 //
-//   * persistent blocks, one per SM, each walking (kx, 16-ky) column tiles;
+//   * persistent blocks, one per SM, each walking (kx, 16-ky) column tiles
+//     (or two fields or one of a tile, mac_tma_fields);
 //   * the last warp is the producer: one lane issues bulk copies
 //     (cp.async.bulk) into two rings of shared-memory stages, one for the
 //     entries' kernel tiles (M rows x 128 B, or 64 B for a real kernel) and
@@ -159,8 +160,8 @@ __device__ __forceinline__ void named_sync(int id, int threads)
 // warps between the stages), then rows z < nz (row z of the transform sits at
 // tile_row(z)) to T2.
 template <int M, int NF>
-__device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw, const InvTarget &T, int kxi, int ky0,
-                                                  int f0, int w, int nw, int lane, int bar)
+__device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw, const InvTarget &T, int local, int f0,
+                                                  int w, int nw, int lane, int bar)
 {
     constexpr int B = M / 16, FS = M * kTileY;
     const int tid = w * 32 + lane, nt = nw * 32;
@@ -171,13 +172,13 @@ __device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw,
     named_sync(bar, nt);
     for (int i = tid; i < NF * 256; i += nt) tile_stage2<B, true>(acc + (i >> 8) * FS, i & 15, (i >> 4) & 15);
     named_sync(bar, nt);
-    const int nz = T.nz;
-    const long long t2_field = (long long)(M / 2 + 1) * nz * M;
-    float2 *dst = T.t2 + (long long)f0 * t2_field + (long long)kxi * nz * M + ky0;
+    const int nz = T.nz, my = T.ay.M, nty = my / kTileY, kxi = local / nty, ky0 = (local - kxi * nty) * kTileY;
+    const long long t2_field = (long long)T.kx * nz * my;
+    float2 *dst = T.t2 + (long long)f0 * t2_field + (long long)kxi * nz * my + ky0;
     for (int i = tid; i < NF * nz * (kTileY / 2); i += nt) {
         const int f = i / (nz * (kTileY / 2)), rem = i - f * nz * (kTileY / 2);
         const int zi = rem >> 3, pp = rem & 7;
-        *reinterpret_cast<float4 *>(dst + f * t2_field + (long long)zi * M + 2 * pp) =
+        *reinterpret_cast<float4 *>(dst + f * t2_field + (long long)zi * my + 2 * pp) =
             *reinterpret_cast<const float4 *>(acc + f * FS + tile_row<B>(zi) * kTileY + 2 * pp);
     }
 }
@@ -187,21 +188,23 @@ __device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw,
 template <bool COMP>
 __host__ __device__ constexpr int fft_warps() { return COMP ? 3 : kFftWarps; }
 
-// Field groups per tile: the compensated MAC at M = 192 would hold 128
-// accumulator and compensation floats per MAC thread for all four fields (and
-// spill them), so it sums the tile in two passes of two fields each, every
-// pass over all the tile's entries (the kernel tile read again, mostly from
-// L2), and hands each pass's two fields to the FFT warps on its own.
-__host__ __device__ constexpr int field_groups(int M, bool comp) { return comp && M == 192 ? 2 : 1; }
+// A block's unit of work is FH fields of one tile: all four (the kernel tile
+// read once), unless
+//   * M = 192, compensated: a MAC thread would hold 128 floats of sums and
+//     compensation for four fields and spill them, so a unit is two;
+//   * the plan's tiles are so few that half of the SMs would have none
+//     (elongated and small grids): two fields or one, the kernel tile then
+//     read again from L2 by the neighbouring block (mac_tma_fields).
+// Every field is summed in the same order whatever the unit.
 
-// M: padded FFT size of the class; CW: multiply-accumulate warps (the block
-// has CW + fft_warps + 1); FPC: field tiles per ring copy (1, 2 or 4; they
-// are contiguous in the ring); COMP: the sum over (source, lag) entries is
-// Kahan-compensated per spectral coefficient (the default; RP_FLAG_PLAIN_SUM
-// selects the plain chain).
-template <int M, int CW, int FPC, bool COMP>
+// M: padded FFT size along z; CW: multiply-accumulate warps (the block has
+// CW + fft_warps + 1); FPC: field tiles per ring copy (1, 2 or 4; they are
+// contiguous in the ring); FH: fields of a unit; COMP: the sum over (source,
+// lag) entries is Kahan-compensated per spectral coefficient (the default;
+// RP_FLAG_PLAIN_SUM selects the plain chain).
+template <int M, int CW, int FPC, int FH, bool COMP>
 __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
-    k_mac_tma(const InvTarget *__restrict__ tgts, int t0, int t1, int tile_lo, int ntiles,
+    k_mac_tma(const InvTarget *__restrict__ tgts, int t0, int t1, int tile_lo, int nunits,
               const MacEntry *__restrict__ entries, long long step, int clamp, int ns, int *err)
 {
     constexpr int STAGE = M * 128;                  // one M x 16 complex tile
@@ -211,11 +214,9 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
     constexpr int FW = fft_warps<COMP>();
     constexpr int RSTEP = kConsumerWarps * 32 / 8;   // rows covered by one pass of the consumers
     constexpr int ROWS = (M + RSTEP - 1) / RSTEP;
-    constexpr int NTY = M / kTileY;
     constexpr int FS = M * kTileY;                   // float2 per field of the FFT tile (dense rows)
-    constexpr int NFG = field_groups(M, COMP);      // passes per tile
-    constexpr int FH = 4 / NFG;                      // fields per pass
-    static_assert(FH % FPC == 0, "k_mac_tma: whole field copies per pass");
+    constexpr int NFG = 4 / FH;                      // units per tile: unit u is fields FH (u % NFG) .. of tile u / NFG
+    static_assert(FH % FPC == 0, "k_mac_tma: whole field copies per unit");
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char *sstages = smem;                                   // [ns][SSTAGE]
     unsigned char *gstages = smem + (size_t)ns * SSTAGE;             // [NG][STAGE]
@@ -278,14 +279,13 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
             }
             return true;
         };
-        for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-            const int b = tile + tile_lo;
+        for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+            const int b = u / NFG + tile_lo, h = u % NFG;
             const InvTarget &T = tgts[owner(tgts, t0, t1, b, &InvTarget::tile0)];
             const long long tile_off = (long long)(b - T.tile0) * M * kTileY;
             const int nr = T.er - T.e0, nc = T.e1 - T.er;   // real (self) entries come first
-            for (int k = 0; k < NFG * (nr + nc) && ok; ++k) {   // pass h = k / (nr + nc) of the tile
-                const int h = k / (nr + nc);
-                const MacEntry &E = entries[T.e0 + k - h * (nr + nc)];
+            for (int k = 0; k < nr + nc && ok; ++k) {
+                const MacEntry &E = entries[T.e0 + k];
                 long long j = step - E.lag;
                 if (clamp && j < 0) j = 0;
                 const int slot = (int)(j % E.depth);
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
                     bulk_load(gstages + (size_t)s * STAGE, src, bytes, &gfull[s], keep);
                     ++qg;
                 }
-                // the pass's field tiles of the source spectrum (fields h FH ..), FPC per copy
+                // the unit's field tiles of the source spectrum (fields h FH ..), FPC per copy
                 const float2 *fields = E.ring + (long long)slot * E.slot_elems + 4 * tile_off;
                 for (int o = 0; o < FH / FPC; ++o) {
                     if (!(ok = acquire(sempty, ns, qs))) break;
@@ -320,37 +320,33 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
         return;
     }
 
-    // Hand-over, per pass of a tile (one pass of all four fields, or two of
-    // two): the MAC warps accumulate the pass in registers, store it to the
-    // FFT tile and signal accfull; the FFT warps transform and store it while
-    // the MAC warps accumulate the next pass, then signal accempty.  A
-    // block's last pass has no successor, so all its consumer warps share
+    // Hand-over, per unit: the MAC warps accumulate it in registers, store it
+    // to the FFT tile and signal accfull; the FFT warps transform and store it
+    // while the MAC warps accumulate the next, then signal accempty.  A
+    // block's last unit has no successor, so all its consumer warps share
     // that transform (barrier 2 in place of the two signals).
     constexpr int kBarFft = 1, kBarAll = 2;
     if (warp >= kConsumerWarps) {
         // ------------------------------------------------------------ FFT warps
         const int fw = warp - kConsumerWarps;
         uint32_t it = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            const int b = tile + tile_lo;
+        for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++it) {
+            const int b = u / NFG + tile_lo, h = u % NFG;
             const InvTarget &T = tgts[owner(tgts, t0, t1, b, &InvTarget::tile0)];
-            const int local = b - T.tile0, kxi = local / NTY, ky0 = (local % NTY) * kTileY;
-            for (int h = 0; h < NFG; ++h, ++it) {
-                if (tile + (int)gridDim.x >= ntiles && h == NFG - 1) {
-                    named_sync(kBarAll, (kConsumerWarps + FW) * 32);
-                    column_tile_store<M, FH>(acc, tw, T, kxi, ky0, h * FH, warp, kConsumerWarps + FW, lane, kBarAll);
-                    return;
-                }
-                const bool have = wait_or_abort(accfull, it & 1);
-                // on an abort the sums are not used: skip the transform, keep the barriers
-                if (have) column_tile_store<M, FH>(acc, tw, T, kxi, ky0, h * FH, fw, FW, lane, kBarFft);
-                else {
-                    named_sync(kBarFft, FW * 32);
-                    named_sync(kBarFft, FW * 32);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(accempty);
+            if (u + (int)gridDim.x >= nunits) {
+                named_sync(kBarAll, (kConsumerWarps + FW) * 32);
+                column_tile_store<M, FH>(acc, tw, T, b - T.tile0, h * FH, warp, kConsumerWarps + FW, lane, kBarAll);
+                return;
             }
+            const bool have = wait_or_abort(accfull, it & 1);
+            // on an abort the sums are not used: skip the transform, keep the barriers
+            if (have) column_tile_store<M, FH>(acc, tw, T, b - T.tile0, h * FH, fw, FW, lane, kBarFft);
+            else {
+                named_sync(kBarFft, FW * 32);
+                named_sync(kBarFft, FW * 32);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(accempty);
         }
         return;
     }
@@ -369,10 +365,10 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
         if (lane == 0) mbar_arrive(&empty[q % n]);
     };
 
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int b = tile + tile_lo;
+    for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++it) {
+        const int b = u / NFG + tile_lo, h = u % NFG;
         const InvTarget &T = tgts[owner(tgts, t0, t1, b, &InvTarget::tile0)];
-        for (int h = 0; h < NFG; ++h, ++it) {   // pass h: fields h FH .. h FH + FH - 1
+        {   // fields h FH .. h FH + FH - 1
             float4 a[ROWS][FH];
             float4 cmp[COMP ? ROWS : 1][FH];   // Kahan compensation (COMP only)
 #pragma unroll
@@ -467,7 +463,7 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
                 }
             }
 
-            // hand the sums to the FFT warps once they are done with the previous pass
+            // hand the sums to the FFT warps once they are done with the previous unit
             if (it == 0 || wait_or_abort(accempty, (it - 1) & 1)) {
 #pragma unroll
                 for (int i = 0; i < ROWS; ++i) {
@@ -483,11 +479,9 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
                     }
                 }
             }
-            if (tile + (int)gridDim.x >= ntiles && h == NFG - 1) {
+            if (u + (int)gridDim.x >= nunits) {
                 named_sync(kBarAll, (kConsumerWarps + FW) * 32);
-                const int local = b - T.tile0;
-                column_tile_store<M, FH>(acc, tw, T, local / NTY, (local % NTY) * kTileY, h * FH, warp,
-                                         kConsumerWarps + FW, lane, kBarAll);
+                column_tile_store<M, FH>(acc, tw, T, b - T.tile0, h * FH, warp, kConsumerWarps + FW, lane, kBarAll);
                 return;
             }
             __syncwarp();
@@ -496,8 +490,28 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
     }
 }
 
-// (class, field tiles per ring copy): must match mac_tma_fields_per_copy
-#define RP_TMA_CLASSES(X) X(32, 4) X(48, 4) X(64, 4) X(96, 4) X(128, 2) X(192, 1)
+constexpr int fields_per_copy(int M, int fh)
+{
+    const int f = M <= 96 ? 4 : (M == 128 ? 2 : 1);
+    return f < fh ? f : fh;
+}
+
+// every (class, fields of a unit) that runs: M = 192, compensated, has no unit of four
+#define RP_TMA_CLASSES(X) X(32) X(48) X(64) X(96) X(128) X(192)
+#define RP_TMA_FIELDS(X, M) X(M, 4) X(M, 2) X(M, 1)
+constexpr bool unit_runs(int M, int fh, bool comp) { return !(comp && M == 192 && fh == 4); }
+
+template <int M, int FH, class F>
+cudaError_t for_variants(F &&f)   // f(kernel, consumer warps, compensated)
+{
+    constexpr int FPC = fields_per_copy(M, FH);
+    cudaError_t e;
+    if ((e = f(k_mac_tma<M, 8, FPC, FH, false>, 8, false)) || (e = f(k_mac_tma<M, 12, FPC, FH, false>, 12, false)) ||
+        (e = f(k_mac_tma<M, 16, FPC, FH, false>, 16, false)))
+        return e;
+    if constexpr (unit_runs(M, FH, true)) return f(k_mac_tma<M, kCompWarps, FPC, FH, true>, kCompWarps, true);
+    return cudaSuccess;
+}
 
 }  // namespace
 
@@ -507,68 +521,75 @@ cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_
     return cudaGetLastError();
 }
 
-int mac_tma_fields_per_copy(int M) { return M <= 96 ? 4 : (M == 128 ? 2 : 1); }
-
-int mac_tma_stages(int M, int smem_optin, bool comp)
+// Fields of a unit: as many as the registers hold, halved while the units
+// would still not outnumber the SMs: a block alone reads about 1/152 of the
+// HBM bandwidth, so idle SMs cost it.  Two 16 x 16 x 60 boxes (68 tiles of M =
+// 128, 40 entries): 54.7 us per step with four fields, 44.2 with two; one 8 x
+// 8 x 90 box (17 tiles of M = 192): 40.3 with two, 33.5 with one.  Beyond one
+// unit per SM the shorter copies only cost (16 x 16 x 96 pair: 67.7 with two,
+// 80.6 with one).
+int mac_tma_fields(int M, bool comp, int ntiles, int sms)
 {
-    const long long sstage = (long long)mac_tma_fields_per_copy(M) * M * 128;
-    const long long fixed = (long long)mac_tma_smem(M, 0, comp);   // kernel-tile ring, FFT tile, twiddles, barriers
+    int fh = unit_runs(M, 4, comp) ? 4 : 2;
+    while (fh > 1 && ntiles * (4 / fh) * 2 <= sms) fh /= 2;
+    return fh;
+}
+
+int mac_tma_stages(int M, int smem_optin, int fh)
+{
+    const long long sstage = (long long)fields_per_copy(M, fh) * M * 128;
+    const long long fixed = (long long)mac_tma_smem(M, 0, fh);   // kernel-tile ring, FFT tile, twiddles, barriers
     long long n = (smem_optin - fixed) / (sstage + 16);      // + two mbarriers per stage
     if (n > kMaxStages) n = kMaxStages;
     return (int)n;
 }
 
-size_t mac_tma_smem(int M, int nstages, bool comp)
+size_t mac_tma_smem(int M, int nstages, int fh)
 {
-    const size_t stage = (size_t)M * 128, fields = 4 / field_groups(M, comp);   // fields of the FFT tile
-    return (size_t)nstages * mac_tma_fields_per_copy(M) * stage + kKernelStages * stage +
-           sizeof(float2) * (fields * (size_t)M * kTileY + M) + 16 * ((size_t)nstages + kKernelStages) + 16 + 16;
+    const size_t stage = (size_t)M * 128;
+    return (size_t)nstages * fields_per_copy(M, fh) * stage + kKernelStages * stage +
+           sizeof(float2) * (fh * (size_t)M * kTileY + M) + 16 * ((size_t)nstages + kKernelStages) + 16 + 16;
 }
 
 cudaError_t open_mac_tma_smem_limit(int max_optin)
 {
     cudaError_t e;
-#define X(M, F)                                                                                                   \
-    if ((e = cudaFuncSetAttribute(k_mac_tma<M, 8, F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                  max_optin)) ||                                                                  \
-        (e = cudaFuncSetAttribute(k_mac_tma<M, 12, F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                                  max_optin)) ||                                                                  \
-        (e = cudaFuncSetAttribute(k_mac_tma<M, 16, F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                                  max_optin)) ||                                                                  \
-        (e = cudaFuncSetAttribute(k_mac_tma<M, kCompWarps, F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                  max_optin)))                                                                    \
-        return e;
-    RP_TMA_CLASSES(X)
+    const auto open = [&](auto kern, int, bool) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
+    };
+#define X(M, FH) \
+    if ((e = for_variants<M, FH>(open))) return e;
+#define Y(M) RP_TMA_FIELDS(X, M)
+    RP_TMA_CLASSES(Y)
+#undef Y
 #undef X
     return cudaSuccess;
 }
 
 cudaError_t launch_mac_tma(int cls, int cw, bool comp, const InvTarget *d_tgts, int t0, int t1, int tile_lo,
-                           int ntiles, const MacEntry *d_entries, long long step, int clamp, int nstages, int grid,
-                           int *d_err, cudaStream_t s)
+                           int ntiles, const MacEntry *d_entries, long long step, int clamp, int fh, int nstages,
+                           int sms, int *d_err, cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
     if (comp ? cw != kCompWarps : (cw != 8 && cw != 12 && cw != 16)) return cudaErrorInvalidValue;
-    if (nstages < 2 || nstages > kMaxStages) return cudaErrorInvalidValue;
-    const size_t smem = mac_tma_smem(cls, nstages, comp);
+    if (nstages < 2 || nstages > kMaxStages || (fh != 4 && fh != 2 && fh != 1) || !unit_runs(cls, fh, comp))
+        return cudaErrorInvalidValue;
+    const size_t smem = mac_tma_smem(cls, nstages, fh);
     const int threads = (cw + (comp ? fft_warps<true>() : fft_warps<false>()) + 1) * 32;
-    cudaError_t e = cudaSuccess;
-#define RP_GO(M, CW, F, C)                                                                                   \
-    e = launch_pdl(k_mac_tma<M, CW, F, C>, dim3(grid), dim3(threads), smem, s, d_tgts, t0, t1, tile_lo, ntiles, \
-                   d_entries, step, clamp, nstages, d_err)
-    switch (cls) {
-#define X(M, F)                                                                                         \
-    case M:                                                                                             \
-        if (comp) RP_GO(M, kCompWarps, F, true);                                                        \
-        else if (cw == 8) RP_GO(M, 8, F, false);                                                        \
-        else if (cw == 12) RP_GO(M, 12, F, false);                                                      \
-        else RP_GO(M, 16, F, false);                                                                    \
-        break;
-        RP_TMA_CLASSES(X)
+    const int nunits = ntiles * (4 / fh), grid = nunits < sms ? nunits : sms;
+    cudaError_t e = cudaErrorInvalidValue;
+    const auto go = [&](auto kern, int w, bool c) {
+        if (w == cw && c == comp)
+            e = launch_pdl(kern, dim3(grid), dim3(threads), smem, s, d_tgts, t0, t1, tile_lo, nunits, d_entries, step,
+                           clamp, nstages, d_err);
+        return cudaSuccess;
+    };
+#define X(M, FH) \
+    if (cls == M && fh == FH) for_variants<M, FH>(go);
+#define Y(M) RP_TMA_FIELDS(X, M)
+    RP_TMA_CLASSES(Y)
+#undef Y
 #undef X
-    default: return cudaErrorInvalidValue;
-    }
-#undef RP_GO
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
