@@ -1009,15 +1009,6 @@ rp_status rp_finalize(rp_ctx *ctx)
     });
     std::vector<int> ring_pos(ring_keys.size());
     std::map<int, const float2 *> tw;
-    {   // the plane passes' form per class, from its forward plane blocks
-        int blocks[7] = {};
-        for (size_t r = 0; r < ring_keys.size(); ++r)
-            blocks[class_slot(plane_class(ring_class((int)r)))] += 4 * ctx->doms[ring_keys[r].first].n[2];
-        for (size_t r = 0; r < ring_keys.size(); ++r) {
-            const int cls = plane_class(ring_class((int)r));
-            ctx->fwd_tile[class_slot(cls)] = plane_tile_form(cls, blocks[class_slot(cls)], false);
-        }
-    }
     for (size_t i = 0; i < ring_order.size(); ++i) {
         const int r = ring_order[i];
         ring_pos[r] = (int)i;
@@ -1040,7 +1031,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         ctx->spec_depth = std::max(ctx->spec_depth, R.depth);
         {
             const int c = plane_class(size_class(R.ax, R.ay, R.az)), cs = class_slot(c);
-            const size_t need = smem_fwd_plane(c, ctx->fwd_tile[cs], R.ny, R.ax);
+            const size_t need = smem_fwd_plane(c, R.ny, R.ax);
             ctx->smem_plane_cls[cs] = std::max(ctx->smem_plane_cls[cs], need);
             ctx->smem_plane = std::max(ctx->smem_plane, need);
         }
@@ -1068,14 +1059,6 @@ rp_status rp_finalize(rp_ctx *ctx)
     };
     std::stable_sort(tgt_order.begin(), tgt_order.end(),
                      [&](int x, int y) { return tgt_class(x) < tgt_class(y); });
-    {   // the inverse plane pass's form per class, from its blocks
-        int blocks[7] = {};
-        for (int t : tgt_order) blocks[class_slot(plane_class(tgt_class(t)))] += 4 * ctx->doms[t].n[2];
-        for (int t : tgt_order) {
-            const int cls = plane_class(tgt_class(t));
-            ctx->inv_tile[class_slot(cls)] = plane_tile_form(cls, blocks[class_slot(cls)], true);
-        }
-    }
     for (int t : tgt_order) {
         const DomainDesc &T = ctx->doms[t];
         InvTarget I{};
@@ -1118,7 +1101,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         ctx->smem_mac = std::max(ctx->smem_mac, smem_mac_inv_column(I.az));
         {
             const int c = plane_class(size_class(I.ax, I.ay, I.az)), cs = class_slot(c);
-            const size_t need = smem_inv_plane(c, ctx->inv_tile[cs], I.nx, I.ny, I.ax, I.ay);
+            const size_t need = smem_inv_plane(c, I.nx, I.ny, I.ax, I.ay);
             ctx->smem_inv_cls[cs] = std::max(ctx->smem_inv_cls[cs], need);
             ctx->smem_inv = std::max(ctx->smem_inv, need);
         }
@@ -1513,8 +1496,7 @@ rp_status enqueue_push(rp_ctx *ctx, int d0, int d1, const IoPtrs &in)
     for (const LaunchGroup &g : launches) {
         const int cls = plane_class(g.cls);
         if ((st = timed_launch(ctx, RP_K_FWD_PLANE, "forward plane pass", [&] {
-                 return launch_fwd_plane(cls, ctx->fwd_tile[class_slot(cls)], rings, fin, g.i0, g.i1, g.blk0,
-                                         g.blk1 - g.blk0, ctx->smem_plane_cls[class_slot(cls)],
+                 return launch_fwd_plane(cls, rings, fin, g.i0, g.i1, g.blk0, g.blk1 - g.blk0, ctx->smem_plane_cls[class_slot(cls)],
                                          (int)(step % std::max(1, ctx->cfg.far_batch)), ctx->stream);
              })))
             return st;
@@ -1946,8 +1928,7 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
     for (const LaunchGroup &g : ctx->inv_groups) {
         const int cls = plane_class(g.cls);
         if ((st = timed_launch(ctx, RP_K_INV_PLANE, "inverse plane pass", [&] {
-                 return launch_inv_plane(cls, ctx->inv_tile[class_slot(cls)], ctx->d_inv, g.i0, g.i1, g.blk2_0,
-                                         out, g.blk2_1 - g.blk2_0, ctx->smem_inv_cls[class_slot(cls)], inv_c, kstep,
+                 return launch_inv_plane(cls, ctx->d_inv, g.i0, g.i1, g.blk2_0, out, g.blk2_1 - g.blk2_0, ctx->smem_inv_cls[class_slot(cls)], inv_c, kstep,
                                          ctx->stream);
              })))
             return st;

@@ -166,8 +166,7 @@ struct rp_ctx {
     size_t smem_plane = 0, smem_col = 0, smem_mac = 0, smem_inv = 0;
     int dir_nlag = 0, dir_splits = 1;                // direct sums: longest lag window, parts of the sources
     float *dir_part = nullptr;                       // their workspace (more than one part)
-    bool fwd_tile[7] = {}, inv_tile[7] = {};            // plane-pass form per class (index by class_slot)
-    size_t smem_plane_cls[7] = {}, smem_inv_cls[7] = {}; // their shared memory per launch
+    size_t smem_plane_cls[7] = {}, smem_inv_cls[7] = {}; // plane passes' shared memory per launch (by class_slot)
     int max_lag = 0, raw_depth = 0, spec_depth = 0;
     long long spectral_bytes = 0, kernel_bytes = 0, device_bytes = 0;
 

@@ -437,27 +437,6 @@ __device__ __forceinline__ void tile_fft16_pair(float2 *T, const float2 *tw, int
     asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
 }
 
-// ntiles tiles (tile i at T + i * tile_stride) by the whole block, the tasks
-// of each stage spread over its threads (16 consecutive threads take the 16
-// lines of one row); ends with the block synchronised.
-template <int B, bool INV, bool HALF, int SP, int SC>
-__device__ __forceinline__ void tiles_fft_block(float2 *T, int tile_stride, int ntiles, const float2 *tw, int nin)
-{
-    const int n1 = ntiles * 16 * B;
-#pragma unroll 1
-    for (int i = threadIdx.x; i < n1; i += blockDim.x) {
-        const int c = i & 15, rest = i >> 4;
-        const int tile = rest / B, n2 = rest - tile * B;
-        tile_stage1<B, INV, HALF, SP, SC>(T + tile * tile_stride, tw, nin, c, n2);
-    }
-    __syncthreads();
-    const int n2t = ntiles * 256;
-#pragma unroll 1
-    for (int i = threadIdx.x; i < n2t; i += blockDim.x)
-        tile_stage2<B, INV, SP, SC>(T + (i >> 8) * tile_stride, i & 15, (i >> 4) & 15);
-    __syncthreads();
-}
-
 // Runtime dispatch on R for a functor templated on R:  f.template run<R>().
 template <class F>
 __device__ __forceinline__ void dispatch_radix(int R, F &f)

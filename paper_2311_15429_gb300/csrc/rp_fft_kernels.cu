@@ -14,13 +14,12 @@
 // the scratch after a plane pass is [field][kx][z][ky]; every field array of
 // a domain is [z][y][x].
 //
-// The passes come in two forms.  k_fwd_plane16, k_fwd_column16 and
-// k_inv_plane16 run the two-stage shared-memory tile transform of rp_fft.cuh
-// (M = 16 B: the plane passes for M = 64, 96, 128, the column pass also for
-// 192).  k_fwd_plane, k_fwd_column and k_inv_plane run the lane-shuffle line
-// transform for the other sizes (32, 48, and 192 for the plane passes) and for
-// M = 0 (any supported shape, read at run time).  The MAC here serves shapes
-// with no column class.
+// The column pass runs the two-stage shared-memory tile transform of
+// rp_fft.cuh for 64, 96, 128 and 192 points along z (k_fwd_column16) and the
+// lane-shuffle line transform otherwise; the plane passes here (lane-shuffle
+// lines) serve a cross-section of 48 and, with M = 0, any supported shape read
+// at run time; the other square ones are in rp_plane.cu.  The MAC here serves
+// shapes with no column class.
 #include <cuda_runtime.h>
 
 #include "rp_fft.cuh"
@@ -712,372 +711,10 @@ __global__ void __launch_bounds__(kPlaneThreads) k_inv_plane(const InvTarget *__
     }
 }
 
-// ---------------------------------------------------------------- plane passes on tiles (M = 64, 96, 128)
-//
-// The plane passes on the two-stage tile transform.  Forward: the plane's
-// rows in pairs (row 2c the real part of line c, row 2c + 1 the imaginary
-// part) transformed along x as row lines, split into the two rows' spectra
-// (Z[k] +- conj Z[M-k]), then along y as column lines over kx.  The columns
-// kx = 0 and kx = M/2 of a real plane are real, so they travel as one
-// complex column (kx = 0 in the real part, M/2 in the imaginary part) and are
-// split after the y transform: the y pass is M/32 whole tiles.  Inverse: the
-// same steps in reverse order, the rows kx = 0 and M/2 packed as S_0 + i S_M/2
-// (their transforms along y are real up to rounding), and the C2R transform
-// along x as one complex transform per pair of output rows.  A class runs
-// these while its planes fit in about one wave (plane_tile_form: 3 blocks of
-// 256 threads per SM); over many waves the lane-shuffle passes, with twice
-// the blocks per SM, finish first.
-constexpr int kPlane16Threads = 256;
-
-__host__ __device__ constexpr bool plane16_class(int M) { return M == 64 || M == 96 || M == 128; }
-__host__ __device__ constexpr int plane16_xtiles(int ny) { return ((ny + 1) / 2 + 15) / 16; }
-
-// 4-byte asynchronous global -> shared copy
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
-                 : "memory");
-}
-// 8-byte asynchronous global -> shared copy
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
-                 : "memory");
-}
-
-template <int M>
-__global__ void __launch_bounds__(kPlane16Threads, 3) k_fwd_plane16(const FwdRing *__restrict__ rings, IoPtrs in, int r0,
-                                                                 int r1, int block_lo, int far_slot)
-{
-    constexpr int B = M / 16, H = M / 2, SX = M + 1, SQ = H + 1;
-    static_assert(plane16_class(M), "k_fwd_plane16: M = 64, 96 or 128");
-    extern __shared__ float4 smem_f4[];
-    float2 *sm = reinterpret_cast<float2 *>(smem_f4);
-    const int b = blockIdx.x + block_lo;
-    const int r = owner_of(rings, r0, r1, b, &FwdRing::plane0);
-    const FwdRing &R = rings[r];
-    const int nx = R.nx, ny = R.ny, nz = R.nz;
-    const int local = b - R.plane0;
-    const int f = local / nz, z = local % nz;
-    const long long N = (long long)nx * ny * nz;
-    const int pairs = (ny + 1) >> 1, xt = (pairs + 15) >> 4;
-    float2 *twx = sm, *twy = sm + M;
-    float2 *X = twy + M;            // x pass: line c (rows 2c, 2c + 1) at X + c * SX
-    float2 *Q = X + xt * 16 * SX;   // y pass: [M rows y][SQ]; column 0 = kx 0 and H, column k = kx k
-    load_twiddles(twx, R.tw_x, M);
-    load_twiddles(twy, R.tw_y, M);
-    pdl_trigger();
-    pdl_wait();   // the input slice may come from the previous kernel; t1 was read by it
-    const float *src = f == 0 ? in.rho[R.src] : in.J[R.src] + (long long)(f - 1) * N;
-    const float *plane = src + (long long)z * nx * ny;
-    float *Xf = reinterpret_cast<float *>(X);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int y = warp; y < ny; y += nwarps)
-        for (int x = lane; x < nx; x += 32) cp_async4(Xf + 2 * ((y >> 1) * SX + x) + (y & 1), plane + y * nx + x);
-    if (ny & 1)
-        for (int x = threadIdx.x; x < nx; x += blockDim.x) Xf[2 * ((ny >> 1) * SX + x) + 1] = 0.0f;
-    cp_async_wait_all();
-    __syncthreads();
-    if (nx <= H) tiles_fft_block<B, false, true, 1, SX>(X, 16 * SX, xt, twx, nx);
-    else tiles_fft_block<B, false, false, 1, SX>(X, 16 * SX, xt, twx, nx);
-    // two real rows from one complex transform:
-    //   A[k] = (Z[k] + conj Z[M-k]) / 2,  B[k] = (Z[k] - conj Z[M-k]) / (2i)
-    for (int i = threadIdx.x; i < pairs * H; i += blockDim.x) {
-        const int c = i / H, k = i - c * H;
-        const float2 *L = X + c * SX;
-        const int ya = 2 * c, yb = ya + 1;
-        if (k == 0) {
-            const float2 z0 = L[tile_row<B>(0)], zh = L[tile_row<B>(H)];
-            Q[ya * SQ] = make_float2(z0.x, zh.x);
-            if (yb < ny) Q[yb * SQ] = make_float2(z0.y, zh.y);
-        } else {
-            const float2 zk = L[tile_row<B>(k)], zc = cconj(L[tile_row<B>(M - k)]);
-            const float2 D = csub(zk, zc);
-            Q[ya * SQ + k] = cscale(cadd(zk, zc), 0.5f);
-            if (yb < ny) Q[yb * SQ + k] = make_float2(0.5f * D.y, -0.5f * D.x);
-        }
-    }
-    __syncthreads();
-    if (ny <= H) tiles_fft_block<B, false, true, SQ, 1>(Q, 16, H / 16, twy, ny);
-    else tiles_fft_block<B, false, false, SQ, 1>(Q, 16, H / 16, twy, ny);
-    // rows kx of T1 (ky natural), kx = 0 and H split from the packed column
-    float2 *out = R.t1 + ((long long)f * (H + 1) * nz + z) * M;
-    const long long rs = (long long)nz * M;
-    for (int kxi = warp; kxi <= H; kxi += nwarps) {
-        float2 *row = out + kxi * rs;
-        if (kxi > 0 && kxi < H) {
-            for (int ky = 2 * lane; ky < M; ky += 64) {
-                const float2 a = Q[tile_row<B>(ky) * SQ + kxi], c = Q[tile_row<B>(ky + 1) * SQ + kxi];
-                *reinterpret_cast<float4 *>(row + ky) = make_float4(a.x, a.y, c.x, c.y);
-            }
-        } else {
-            for (int ky = lane; ky < M; ky += 32) {
-                const float2 zk = Q[tile_row<B>(ky) * SQ], zc = cconj(Q[tile_row<B>(ky == 0 ? 0 : M - ky) * SQ]);
-                const float2 D = csub(zk, zc);
-                row[ky] = kxi == 0 ? cscale(cadd(zk, zc), 0.5f) : make_float2(0.5f * D.y, -0.5f * D.x);
-            }
-        }
-    }
-    if (R.far_x) {
-        // far path: this plane as bf16 hi/lo into row (slot, field) of the batch matrix
-        __nv_bfloat16 *row = R.far_x + ((long long)far_slot * 4 + f) * 2 * R.far_ks + (long long)z * nx * ny;
-        for (int i = threadIdx.x; i < nx * ny; i += blockDim.x) {
-            const float v = __ldg(plane + i);
-            const __nv_bfloat16 hi = __float2bfloat16(v);
-            row[i] = hi;
-            row[R.far_ks + i] = __float2bfloat16(v - __bfloat162float(hi));
-        }
-    }
-}
-
-template <int M>
-__global__ void __launch_bounds__(kPlane16Threads, 3) k_inv_plane16(const InvTarget *__restrict__ tgts, int t0, int t1,
-                                                                 int block_lo, OutPtrs out, float inv_c, long long step)
-{
-    constexpr int B = M / 16, H = M / 2, SP = M + 1, SX = 17;
-    static_assert(plane16_class(M), "k_inv_plane16: M = 64, 96 or 128");
-    extern __shared__ float4 smem_f4[];
-    float2 *sm = reinterpret_cast<float2 *>(smem_f4);
-    const int b = blockIdx.x + block_lo;
-    const int t = owner_of(tgts, t0, t1, b, &InvTarget::plane0);
-    const InvTarget &T = tgts[t];
-    const int nx = T.nx, ny = T.ny, nz = T.nz;
-    const int local = b - T.plane0;
-    const int f = local / nz, z = local % nz;
-    const int pairs = (ny + 1) >> 1, xt = (pairs + 15) >> 4;
-    float2 *twx = sm, *twy = sm + M;
-    float2 *P = twy + M;            // y pass: line kx (row lines, ky along), line 0 = kx 0 and H packed
-    float2 *X = P + H * SP;         // x pass: [xt][M rows k][SX], 16 lines (pairs of output rows) per tile
-    float *O = reinterpret_cast<float *>(P);                  // [ny][nx] output plane (P is dead by then)
-    float *fw = reinterpret_cast<float *>(X + xt * M * SX);   // far weights and scratch
-    load_twiddles(twx, T.tw_x, M);
-    load_twiddles(twy, T.tw_y, M);
-    const FarTarget *Fp = T.far;
-    int fpx = 0, fpy = 0, fpz = 0, fr = 0, fdepth = 1;
-    const float *fcring = nullptr;
-    float *cz = fw;                                         // [py][px]
-    float *ux = cz + kMaxFarPts * kMaxFarPts;               // [py][nx]
-    float *sLx = ux + kMaxFarPts * nx;                      // [nx][px]
-    float *sLy = sLx + kMaxFarPts * nx;                     // [ny][py]
-    float *sLz = sLy + kMaxFarPts * ny;                     // [pz], row z
-    float *sc = sLz + kMaxFarPts;                           // [r]: this step's coefficients of field f
-    if (Fp) {
-        fpx = Fp->px; fpy = Fp->py; fpz = Fp->pz; fr = Fp->r; fdepth = Fp->depth; fcring = Fp->cring;
-        for (int i = threadIdx.x; i < nx * fpx; i += blockDim.x) sLx[i] = __ldg(Fp->Lx + i);
-        for (int i = threadIdx.x; i < ny * fpy; i += blockDim.x) sLy[i] = __ldg(Fp->Ly + i);
-        for (int i = threadIdx.x; i < fpz; i += blockDim.x) sLz[i] = __ldg(Fp->Lz + z * fpz + i);
-    }
-    pdl_trigger();
-    pdl_wait();   // T2 is written by the MAC, the coefficient ring by the far scatter or the learned field
-    if (step < 0) step = *T.d_step;   // graph replay: the step from the device counter
-    const float2 *src = T.t2 + ((long long)f * (H + 1) * nz + z) * M;
-    const long long rs = (long long)nz * M;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int kxi = 1 + warp; kxi < H; kxi += nwarps)
-        for (int ky = lane; ky < M; ky += 32) cp_async8(P + kxi * SP + ky, src + kxi * rs + ky);
-    for (int ky = threadIdx.x; ky < M; ky += blockDim.x) {
-        const float2 a = src[ky], h = src[H * rs + ky];
-        P[ky] = make_float2(a.x - h.y, a.y + h.x);   // S_0 + i S_H
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    tiles_fft_block<B, true, false, 1, SP>(P, 16 * SP, H / 16, twy, M);
-    // x-pass input of the pair (ya, yb): A + iB over k < M, from the rows'
-    // half spectra (kx = 0 and H real: the real and imaginary parts of line 0)
-    for (int c = warp; c < pairs; c += nwarps)
-        for (int k = lane; k < M; k += 32) {
-        const int ya = 2 * c, yb = ya + 1;
-        const bool vb = yb < ny;
-        const int kk = k <= H ? k : M - k;
-        float2 A, Bv;
-        if (kk == 0 || kk == H) {
-            const float2 pa = P[tile_row<B>(ya)], pb = vb ? P[tile_row<B>(yb)] : make_float2(0.0f, 0.0f);
-            A = make_float2(kk == 0 ? pa.x : pa.y, 0.0f);
-            Bv = make_float2(kk == 0 ? pb.x : pb.y, 0.0f);
-        } else {
-            const float2 *L = P + kk * SP;
-            A = L[tile_row<B>(ya)];
-            Bv = vb ? L[tile_row<B>(yb)] : make_float2(0.0f, 0.0f);
-            if (k > H) { A = cconj(A); Bv = cconj(Bv); }
-        }
-        X[(c >> 4) * M * SX + k * SX + (c & 15)] = make_float2(A.x - Bv.y, A.y + Bv.x);
-        }
-    __syncthreads();
-    tiles_fft_block<B, true, false, SX, 1>(X, M * SX, xt, twx, M);
-    const long long Nt = (long long)nx * ny * nz;
-    float *dst = (f == 0 ? out.phi[T.dom] : out.A[T.dom] + (long long)(f - 1) * Nt) + (long long)z * nx * ny;
-    const float scale = f == 0 ? 1.0f : inv_c;
-    float *O_or_dst = Fp ? O : dst;
-    for (int y = warp; y < ny; y += nwarps) {
-        const int c = y >> 1;
-        const float2 *L = X + (c >> 4) * M * SX + (c & 15);
-        for (int x = lane; x < nx; x += 32) {
-            const float2 v = L[tile_row<B>(x) * SX];
-            O_or_dst[y * nx + x] = scale * ((y & 1) ? v.y : v.x);
-        }
-    }
-    if (!Fp) return;
-    // far pairs: tensor-product Lagrange interpolation of this step's node
-    // coefficients (field f), contracted over z first
-    const float *c = fcring + (step % fdepth) * (fr * 4);
-    for (int i = threadIdx.x; i < fr; i += blockDim.x) sc[i] = c[i * 4 + f];
-    __syncthreads();
-    const int pxy = fpx * fpy;
-    for (int i = threadIdx.x; i < pxy; i += blockDim.x) {
-        float s = 0.0f;
-        for (int cc = 0; cc < fpz; ++cc) s = fmaf(sLz[cc], sc[cc * pxy + i], s);
-        cz[i] = s;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < fpy * nx; i += blockDim.x) {
-        const int bb = i / nx, x = i % nx;
-        float u = 0.0f;
-        for (int aa = 0; aa < fpx; ++aa) u = fmaf(sLx[x * fpx + aa], cz[bb * fpx + aa], u);
-        ux[i] = u;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nx * ny; i += blockDim.x) {
-        const int x = i % nx, y = i / nx;
-        float v = 0.0f;
-        for (int bb = 0; bb < fpy; ++bb) v = fmaf(sLy[y * fpy + bb], ux[bb * nx + x], v);
-        dst[i] = fmaf(scale, v, O[i]);
-    }
-}
-
-// ---------------------------------------------------------------- inverse plane pass for M = 192, in chunks
-//
-// At M = 192 a plane of spectra (97 lines of 192) takes 150 KB of shared
-// memory, so the lane-shuffle pass runs one block per SM.  This one runs the
-// tile transform through a single work tile in chunks of 16 lines: along y,
-// 16 kx lines at a time (kx = 0 and M/2 packed as one line, as in
-// k_inv_plane16), keeping only the rows y < ny of each in a compact buffer Y
-// (odd line stride: no bank conflicts); then along x, 16 pairs of output rows
-// at a time, each row written out with the far coefficients' interpolation
-// added (no output plane in shared memory).  About 109 KB per block: two
-// blocks per SM.
-constexpr int kPlaneBigThreads = 256;
-
-__host__ __device__ constexpr int plane_big_ystride(int ny) { return ny | 1; }
-
-template <int M>
-__global__ void __launch_bounds__(kPlaneBigThreads, 2) k_inv_plane_big(const InvTarget *__restrict__ tgts, int t0,
-                                                                       int t1, int block_lo, OutPtrs out, float inv_c,
-                                                                       long long step)
-{
-    constexpr int B = M / 16, H = M / 2, SW = M + 1, SX = 17;
-    static_assert(M == 192, "k_inv_plane_big: M = 192");
-    extern __shared__ float4 smem_f4[];
-    float2 *sm = reinterpret_cast<float2 *>(smem_f4);
-    const int b = blockIdx.x + block_lo;
-    const int t = owner_of(tgts, t0, t1, b, &InvTarget::plane0);
-    const InvTarget &T = tgts[t];
-    const int nx = T.nx, ny = T.ny, nz = T.nz;
-    const int local = b - T.plane0;
-    const int f = local / nz, z = local % nz;
-    const int pairs = (ny + 1) >> 1, SY = plane_big_ystride(ny);
-    float2 *twx = sm, *twy = sm + M;
-    float2 *Y = twy + M;                                  // [H lines][SY]: rows y < ny of the y transform
-    float2 *W = Y + H * SY;                               // work tile: 16 row lines of SW, or M rows of SX
-    float *ux = reinterpret_cast<float *>(W + M * SX);    // far: [py][nx]
-    float *sc = ux + kMaxFarPts * nx;                     // far: [r], this step's coefficients of field f
-    float *cz = sc + kMaxFarPts * kMaxFarPts * kMaxFarPts;   // far: [py][px]
-    load_twiddles(twx, T.tw_x, M);
-    load_twiddles(twy, T.tw_y, M);
-    pdl_trigger();
-    pdl_wait();   // T2 is written by the MAC, the coefficient ring by the far path
-    if (step < 0) step = *T.d_step;   // graph replay: the step from the device counter
-    const float2 *src = T.t2 + ((long long)f * (H + 1) * nz + z) * M;
-    const long long rs = (long long)nz * M;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    __syncthreads();
-    // along y, 16 kx lines per chunk; only the rows y < ny are kept
-    for (int ch = 0; ch < H / 16; ++ch) {
-        for (int l = warp; l < 16; l += nwarps) {
-            const int kxi = 16 * ch + l;
-            float2 *L = W + l * SW;
-            if (kxi == 0) {
-                for (int ky = lane; ky < M; ky += 32) {
-                    const float2 a = src[ky], h = src[H * rs + ky];
-                    L[ky] = make_float2(a.x - h.y, a.y + h.x);   // S_0 + i S_H
-                }
-            } else {
-                for (int ky = lane; ky < M; ky += 32) cp_async8(L + ky, src + kxi * rs + ky);
-            }
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        tiles_fft_block<B, true, false, 1, SW>(W, 16 * SW, 1, twy, M);   // ends synchronised
-        for (int i = threadIdx.x; i < 16 * ny; i += blockDim.x) {
-            const int l = i & 15, y = i >> 4;
-            Y[(16 * ch + l) * SY + y] = W[l * SW + tile_row<B>(y)];
-        }
-        __syncthreads();
-    }
-    // far pairs: this step's node coefficients of field f contracted over z,
-    // then over x (the weights read from global memory)
-    const FarTarget *Fp = T.far;
-    if (Fp) {
-        const int px = Fp->px, py = Fp->py, pz = Fp->pz, r = Fp->r, pxy = px * py;
-        const float *c = Fp->cring + (step % Fp->depth) * (r * 4);
-        for (int i = threadIdx.x; i < r; i += blockDim.x) sc[i] = c[i * 4 + f];
-        __syncthreads();
-        for (int i = threadIdx.x; i < pxy; i += blockDim.x) {
-            float s = 0.0f;
-            for (int cc = 0; cc < pz; ++cc) s = fmaf(__ldg(Fp->Lz + z * pz + cc), sc[cc * pxy + i], s);
-            cz[i] = s;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < py * nx; i += blockDim.x) {
-            const int bb = i / nx, x = i % nx;
-            float u = 0.0f;
-            for (int aa = 0; aa < px; ++aa) u = fmaf(__ldg(Fp->Lx + x * px + aa), cz[bb * px + aa], u);
-            ux[i] = u;
-        }
-    }
-    // along x (C2R), 16 pairs of output rows per chunk
-    const long long Nt = (long long)nx * ny * nz;
-    float *dst = (f == 0 ? out.phi[T.dom] : out.A[T.dom] + (long long)(f - 1) * Nt) + (long long)z * nx * ny;
-    const float scale = f == 0 ? 1.0f : inv_c;
-    for (int c0 = 0; c0 < pairs; c0 += 16) {
-        for (int i = threadIdx.x; i < 16 * M; i += blockDim.x) {
-            const int k = i % M, cc = i / M, c = c0 + cc;
-            float2 v = make_float2(0.0f, 0.0f);
-            if (c < pairs) {
-                const int ya = 2 * c, yb = ya + 1;
-                const bool vb = yb < ny;
-                const int kk = k <= H ? k : M - k;
-                float2 A, Bv;
-                if (kk == 0 || kk == H) {   // the real rows kx = 0 and H: parts of line 0
-                    const float2 pa = Y[ya], pb = vb ? Y[yb] : make_float2(0.0f, 0.0f);
-                    A = make_float2(kk == 0 ? pa.x : pa.y, 0.0f);
-                    Bv = make_float2(kk == 0 ? pb.x : pb.y, 0.0f);
-                } else {
-                    A = Y[kk * SY + ya];
-                    Bv = vb ? Y[kk * SY + yb] : make_float2(0.0f, 0.0f);
-                    if (k > H) { A = cconj(A); Bv = cconj(Bv); }
-                }
-                v = make_float2(A.x - Bv.y, A.y + Bv.x);   // A + iB
-            }
-            W[k * SX + cc] = v;
-        }
-        __syncthreads();
-        tiles_fft_block<B, true, false, SX, 1>(W, M * SX, 1, twx, M);   // ends synchronised
-        const int rows = min(32, ny - 2 * c0);
-        for (int i = threadIdx.x; i < rows * nx; i += blockDim.x) {
-            const int yy = i / nx, x = i - yy * nx, y = 2 * c0 + yy;
-            const float2 v = W[tile_row<B>(x) * SX + (yy >> 1)];
-            float o = scale * ((yy & 1) ? v.y : v.x);
-            if (Fp) {
-                float s = 0.0f;
-                for (int bb = 0; bb < Fp->py; ++bb) s = fmaf(__ldg(Fp->Ly + y * Fp->py + bb), ux[bb * nx + x], s);
-                o = fmaf(scale, s, o);
-            }
-            dst[y * nx + x] = o;
-        }
-        __syncthreads();
-    }
-}
-#define RP_FOR_EACH_CLASS(X) X(0) X(32) X(48) X(64) X(96) X(128) X(192)
+// lengths compiled here: of the plane passes (the others are in rp_plane.cu)
+// and of the column pass
+#define RP_PLANE_CLASSES(X) X(0) X(48)
+#define RP_COLUMN_CLASSES(X) X(0) X(32) X(48) X(64) X(96) X(128) X(192)
 
 }  // namespace
 
@@ -1095,14 +732,9 @@ int size_class(const Axis &ax, const Axis &ay, const Axis &az)
     return column << 8 | plane;
 }
 
-bool plane_tile_class(int size_class) { return plane16_class(size_class); }
-
-size_t smem_fwd_plane(int cls, bool tile, int ny, const Axis &ax)
+size_t smem_fwd_plane(int cls, int ny, const Axis &ax)
 {
-    if (tile && plane16_class(cls)) {
-        const size_t M = cls;
-        return sizeof(float2) * (2 * M + (size_t)plane16_xtiles(ny) * 16 * (M + 1) + M * (M / 2 + 1));
-    }
+    if (plane_line_class(cls)) return smem_fwd_plane_line(cls, ny);
     const int kx = ax.M / 2 + 1;
     const int qs = kx | 1;
     // twiddles (x and y, bounded by kMaxFFT each) + Q + per-group scratch
@@ -1118,18 +750,9 @@ size_t smem_mac_inv_column(const Axis &az)
     return sizeof(float2) * ((size_t)az.M + 4 * (size_t)az.M * kTileYPad);
 }
 
-size_t smem_inv_plane(int cls, bool tile, int nx, int ny, const Axis &ax, const Axis &ay)
+size_t smem_inv_plane(int cls, int nx, int ny, const Axis &ax, const Axis &ay)
 {
-    if (cls == 192) {   // k_inv_plane_big, whatever the form flag
-        const size_t M = 192;
-        return sizeof(float2) * (2 * M + (M / 2) * (size_t)plane_big_ystride(ny) + M * 17) +
-               sizeof(float) * ((size_t)kMaxFarPts * nx + kMaxFarPts * kMaxFarPts * kMaxFarPts + kMaxFarPts * kMaxFarPts);
-    }
-    if (tile && plane16_class(cls)) {
-        const size_t M = cls;
-        return sizeof(float2) * (2 * M + (M / 2) * (M + 1) + (size_t)plane16_xtiles(ny) * M * 17) +
-               sizeof(float) * kMaxFarPts * (kMaxFarPts + 2 * (size_t)nx + ny + 1 + kMaxFarPts * kMaxFarPts);
-    }
+    if (plane_line_class(cls)) return smem_inv_plane_line(cls, nx, ny);
     const int kx = ax.M / 2 + 1;
     const int ps = ay.M | 1;
     // + the far path: coefficients contracted over z, then over x; the
@@ -1141,40 +764,20 @@ size_t smem_inv_plane(int cls, bool tile, int nx, int ny, const Axis &ax, const 
 // The dynamic shared-memory limit is an attribute of the kernel function,
 // shared by every context in the process, so each kernel is opened up to the
 // device's opt-in maximum once (contexts never lower it for one another).
-// Each size class opens the kernels it runs: the tile-transform passes where
-// the class has them, the lane-shuffle passes elsewhere.
-template <int M>
-static cudaError_t open_class_smem(int max_optin)
+cudaError_t open_kernel_smem_limits(int max_optin)
 {
     cudaError_t e;
     const auto open = [&](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                                     max_optin); };
-    if constexpr (plane16_class(M))
-        if ((e = open(k_fwd_plane16<M>)) || (e = open(k_inv_plane16<M>))) return e;
-    if ((e = open(k_fwd_plane<M>))) return e;
-    if constexpr (M == 192) {
-        if ((e = open(k_inv_plane_big<M>))) return e;
-    } else {
-        if ((e = open(k_inv_plane<M>))) return e;
-    }
-    if constexpr (tile16_class(M)) {
-        if ((e = open(k_fwd_column16<M>))) return e;
-    } else {
-        if ((e = open(k_fwd_column<M>))) return e;
-    }
-    return cudaSuccess;
-}
-
-cudaError_t open_kernel_smem_limits(int max_optin)
-{
-    cudaError_t e;
-#define RP_OPEN(M) \
-    if ((e = open_class_smem<M>(max_optin))) return e;
-    RP_FOR_EACH_CLASS(RP_OPEN)
-#undef RP_OPEN
-    for (auto kern : {k_mac_inv_column<false>, k_mac_inv_column<true>})
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin))) return e;
-    return cudaSuccess;
+#define X(M) \
+    if ((e = open(k_fwd_plane<M>)) || (e = open(k_inv_plane<M>))) return e;
+    RP_PLANE_CLASSES(X)
+#undef X
+    if ((e = open(k_fwd_column<0>)) || (e = open(k_fwd_column<32>)) || (e = open(k_fwd_column<48>)) ||
+        (e = open(k_fwd_column16<64>)) || (e = open(k_fwd_column16<96>)) || (e = open(k_fwd_column16<128>)) ||
+        (e = open(k_fwd_column16<192>)) || (e = open(k_mac_inv_column<false>)) || (e = open(k_mac_inv_column<true>)))
+        return e;
+    return open_plane_line_smem(max_optin);
 }
 
 cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, int d1,
@@ -1188,50 +791,21 @@ cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, i
     return cudaGetLastError();
 }
 
-template <int M>
-static cudaError_t launch_fwd_plane_cls(bool tile, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
-                                        int block_lo, int nblocks, size_t smem, int far_slot, cudaStream_t s)
-{
-    if constexpr (plane16_class(M))
-        if (tile)
-            return launch_pdl(k_fwd_plane16<M>, dim3(nblocks), dim3(kPlane16Threads), smem, s, d_rings, in, r0, r1,
-                              block_lo, far_slot);
-    return launch_pdl(k_fwd_plane<M>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_rings, in, r0, r1, block_lo,
-                      far_slot);
-}
-
-template <int M>
-static cudaError_t launch_inv_plane_cls(bool tile, const InvTarget *d_tgts, int t0, int t1, int block_lo,
-                                        const OutPtrs &out, int nblocks, size_t smem, float inv_c, long long step,
-                                        cudaStream_t s)
-{
-    if constexpr (plane16_class(M))
-        if (tile)
-            return launch_pdl(k_inv_plane16<M>, dim3(nblocks), dim3(kPlane16Threads), smem, s, d_tgts, t0, t1,
-                              block_lo, out, inv_c, step);
-    if constexpr (M == 192)
-        return launch_pdl(k_inv_plane_big<M>, dim3(nblocks), dim3(kPlaneBigThreads), smem, s, d_tgts, t0, t1,
-                          block_lo, out, inv_c, step);
-    else
-        return launch_pdl(k_inv_plane<M>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_tgts, t0, t1, block_lo, out,
-                          inv_c, step);
-}
-
-cudaError_t launch_fwd_plane(int cls, bool tile, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
-                             int block_lo, int nblocks, size_t smem, int far_slot, cudaStream_t s)
+cudaError_t launch_fwd_plane(int cls, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1, int block_lo,
+                             int nblocks, size_t smem, int far_slot, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
+    if (plane_line_class(cls))
+        return launch_fwd_plane_line(cls, d_rings, in, r0, r1, block_lo, nblocks, smem, far_slot, s);
     switch (cls) {
-#define X(M)                                                                                                    \
-    case M:                                                                                                     \
-        if (cudaError_t e_ = launch_fwd_plane_cls<M>(tile, d_rings, in, r0, r1, block_lo, nblocks, smem, far_slot, s)) \
-            return e_;                                                                                          \
-        break;
-        RP_FOR_EACH_CLASS(X)
+#define X(M)                                                                                                      \
+    case M:                                                                                                       \
+        return launch_pdl(k_fwd_plane<M>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_rings, in, r0, r1,       \
+                          block_lo, far_slot);
+        RP_PLANE_CLASSES(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <int M>
@@ -1256,7 +830,7 @@ cudaError_t launch_fwd_column(int cls, const FwdRing *d_rings, int r0, int r1, i
         if (cudaError_t e_ = launch_fwd_column_cls<M>(d_rings, r0, r1, block_lo, nblocks, smem, step, s)) \
             return e_;                                                                              \
         break;
-        RP_FOR_EACH_CLASS(X)
+        RP_COLUMN_CLASSES(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }
@@ -1272,21 +846,21 @@ cudaError_t launch_mac_inv_column(bool comp, const InvTarget *d_tgts, int t0, in
                       d_tgts, t0, t1, block_lo, d_entries, step, clamp);
 }
 
-cudaError_t launch_inv_plane(int cls, bool tile, const InvTarget *d_tgts, int t0, int t1, int block_lo,
-                             const OutPtrs &out, int nblocks, size_t smem, float inv_c, long long step, cudaStream_t s)
+cudaError_t launch_inv_plane(int cls, const InvTarget *d_tgts, int t0, int t1, int block_lo, const OutPtrs &out,
+                             int nblocks, size_t smem, float inv_c, long long step, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
+    if (plane_line_class(cls))
+        return launch_inv_plane_line(cls, d_tgts, t0, t1, block_lo, out, nblocks, smem, inv_c, step, s);
     switch (cls) {
-#define X(M)                                                                                                      \
-    case M:                                                                                                       \
-        if (cudaError_t e_ = launch_inv_plane_cls<M>(tile, d_tgts, t0, t1, block_lo, out, nblocks, smem, inv_c, step, s)) \
-            return e_;                                                                                            \
-        break;
-        RP_FOR_EACH_CLASS(X)
+#define X(M)                                                                                                       \
+    case M:                                                                                                        \
+        return launch_pdl(k_inv_plane<M>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_tgts, t0, t1, block_lo,   \
+                          out, inv_c, step);
+        RP_PLANE_CLASSES(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace rp
