@@ -48,8 +48,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-__host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// A complex sum or difference is one packed FP32 instruction on the device
+// (a - b as b * -1 + a: the same one rounding): 12-16 % fewer instructions in
+// the plane passes (forward at M = 192 76 -> 68 us, M = 128 54 -> 51, inverse
+// at M = 96 128 -> 124).  A translation unit that defines RP_SCALAR_COMPLEX
+// keeps two scalar ones: beside the MAC's multiply-add warps the packed form
+// waits for their pipe (32 x 48^3, MAC 380 -> 416 us).
+__host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b)
+{
+#if defined(__CUDA_ARCH__) && !defined(RP_SCALAR_COMPLEX)
+    return __fadd2_rn(a, b);
+#else
+    return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b)
+{
+#if defined(__CUDA_ARCH__) && !defined(RP_SCALAR_COMPLEX)
+    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+#else
+    return make_float2(a.x - b.x, a.y - b.y);
+#endif
+}
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));

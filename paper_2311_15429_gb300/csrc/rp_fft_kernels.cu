@@ -752,7 +752,7 @@ size_t smem_mac_inv_column(const Axis &az)
 
 size_t smem_inv_plane(int cls, int nx, int ny, const Axis &ax, const Axis &ay)
 {
-    if (plane_line_class(cls)) return smem_inv_plane_line(cls, nx, ny);
+    if (plane_line_class(cls)) return smem_inv_plane_line(cls, ny);
     const int kx = ax.M / 2 + 1;
     const int ps = ay.M | 1;
     // + the far path: coefficients contracted over z, then over x; the

@@ -258,7 +258,7 @@ cudaError_t launch_inv_plane(int plane_class, const InvTarget *d_tgts, int t0, i
 // The plane passes of square cross-sections of 32, 64, 96, 128 and 192 points (rp_plane.cu).
 bool plane_line_class(int M);
 size_t smem_fwd_plane_line(int M, int ny);
-size_t smem_inv_plane_line(int M, int nx, int ny);
+size_t smem_inv_plane_line(int M, int ny);
 cudaError_t open_plane_line_smem(int max_optin);
 cudaError_t launch_fwd_plane_line(int M, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1, int block_lo,
                                   int nblocks, size_t smem, int far_slot, cudaStream_t s);

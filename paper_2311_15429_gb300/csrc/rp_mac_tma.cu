@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#define RP_SCALAR_COMPLEX
 #include "rp_fft.cuh"
 #include "rp_internal.h"
 

@@ -28,7 +28,13 @@
 // Shared memory per plane of n = M/2 and the blocks an SM holds: M = 96 39 KB
 // (5), M = 128 70 KB (3), M = 192 109 KB (2); the exchange of the y axis goes
 // in chunks of kx lines to keep it there.
-// @@MEASURED@@
+// Per launch, before (tile and lane-shuffle forms) and now: 32 x 48^3 with far
+// pairs forward 111 -> 93 us, inverse 173 -> 117 (288 MB each: 42 us at the
+// copy rate); 8 x 64^3 92 -> 49 and 125 -> 63 (170 MB: 25 us); 3 x 96^3 100 ->
+// 68 and 188 -> 92 (198 MB: 29 us).  Half of the issue slots are used; what is
+// left is waits on the loads of T2 and on barriers at 24 to 27 warps per SM
+// (prefetching a round of lines, or fewer blocks with more registers, changed
+// nothing or lost).
 #include <cuda_runtime.h>
 
 #include "rp_fft.cuh"
@@ -56,6 +62,8 @@ __host__ __device__ constexpr int inv_row_stride(int M, int ny)
     const int r = M == 128 ? 2 : M / 16, n = ny + (ny & 1);
     return n + ((r - n) % 16 + 16) % 16;
 }
+
+constexpr int kFarRow = kMaxFarPts;   // far coefficients of a row, zero past the target's px
 
 template <class T>
 __device__ __forceinline__ int plane_owner(const T *arr, int lo, int hi, int b)
@@ -300,11 +308,13 @@ __device__ __forceinline__ void inv_lines(const float2 *__restrict__ src, long l
 
 // Along x, 16 first: output row pairs p0 .. p0 + np - 1 (rows 2p real, 2p + 1
 // imaginary part) through E (np lines of 16 B + 1) to the output plane.
-// CROP: nx <= M/2.  far: ux ([py][nx]) interpolated along y onto each value.
+// CROP: nx <= M/2.  far: each row's coefficients vy ([ny][kFarRow]) are
+// interpolated along x onto its values, with the weights lx of this thread's
+// x = k1 + 16 k2 for up to four nodes, read from the table for more.
 template <int M, bool CROP>
 __device__ __forceinline__ void inv_rows(const float2 *Y, int SY, float2 *E, const float2 *tw, int p0, int np, int nx,
-                                         int ny, float scale, const FarTarget *__restrict__ far, const float *ux,
-                                         float *__restrict__ dst)
+                                         int ny, float scale, const FarTarget *__restrict__ far, const float *vy,
+                                         const float4 (&lx)[M / 32], float *__restrict__ dst)
 {
     constexpr int B = M / 16, SE = 16 * B + 1, T = inv_plane_threads(M);
     for (int t = threadIdx.x; t < np * B; t += T) {
@@ -326,7 +336,7 @@ __device__ __forceinline__ void inv_rows(const float2 *Y, int SY, float2 *E, con
         for (int k1 = 1; k1 < 16; ++k1) e[k1] = cmul(v[k1], twid<true>(tw, n2 * k1));
     }
     __syncthreads();
-    const int k1 = threadIdx.x & 15;
+    const int k1 = threadIdx.x & 15, px = far ? far->px : 0;
     for (int p = threadIdx.x >> 4; p < np; p += T / 16) {
         float2 v[B];
 #pragma unroll
@@ -335,24 +345,34 @@ __device__ __forceinline__ void inv_rows(const float2 *Y, int SY, float2 *E, con
         const int ya = 2 * (p0 + p);
         const bool vb = ya + 1 < ny;
         float *row = dst + ya * nx;
+        float4 va = make_float4(0.0f, 0.0f, 0.0f, 0.0f), vc = va;
+        if (far) {
+            va = *reinterpret_cast<const float4 *>(vy + ya * kFarRow);
+            vc = *reinterpret_cast<const float4 *>(vy + (ya + (vb ? 1 : 0)) * kFarRow);
+        }
 #pragma unroll
         for (int k2 = 0; k2 < (CROP ? B / 2 : B); ++k2) {
             const int x = k1 + 16 * k2;
             if (x >= nx) continue;
-            float a = scale * v[k2].x, c = scale * v[k2].y;
+            float a = v[k2].x, c = v[k2].y;
             if (far) {
-                const int py = far->py;
-                float sa = 0.0f, sc = 0.0f;
-                for (int i = 0; i < py; ++i) {
-                    const float u = ux[i * nx + x];
-                    sa = fmaf(__ldg(far->Ly + ya * py + i), u, sa);
-                    if (vb) sc = fmaf(__ldg(far->Ly + (ya + 1) * py + i), u, sc);
+                const float4 l = lx[k2 % (M / 32)];
+                if (CROP && px <= 4) {
+                    a += fmaf(l.w, va.w, fmaf(l.z, va.z, fmaf(l.y, va.y, l.x * va.x)));
+                    c += fmaf(l.w, vc.w, fmaf(l.z, vc.z, fmaf(l.y, vc.y, l.x * vc.x)));
+                } else {
+                    float sa = 0.0f, sc = 0.0f;
+                    for (int i = 0; i < px; ++i) {
+                        const float w = __ldg(far->Lx + x * px + i);
+                        sa = fmaf(w, vy[ya * kFarRow + i], sa);
+                        sc = fmaf(w, vy[(ya + (vb ? 1 : 0)) * kFarRow + i], sc);
+                    }
+                    a += sa;
+                    c += sc;
                 }
-                a = fmaf(scale, sa, a);
-                c = fmaf(scale, sc, c);
             }
-            row[x] = a;
-            if (vb) row[nx + x] = c;
+            row[x] = scale * a;
+            if (vb) row[nx + x] = scale * c;
         }
     }
     __syncthreads();
@@ -373,7 +393,7 @@ __global__ void __launch_bounds__(inv_plane_threads(M), plane_blocks(M))
     const int pairs = (ny + 1) >> 1, SY = inv_row_stride(M, ny);
     float2 *Y = tw + M;                                        // [H + 1][SY]
     float2 *E = Y + (H + 1) * SY;                              // [CH][17 B]
-    float *ux = reinterpret_cast<float *>(E + CH * 17 * B);    // far: [py][nx]
+    float *vy = reinterpret_cast<float *>(E + CH * 17 * B);    // far: [ny][kFarRow]
     load_twiddles(tw, I.tw_x, M);
     float2 w[B];                                               // conj W_M^{n2 k1} of this thread's n2
 #pragma unroll
@@ -388,9 +408,20 @@ __global__ void __launch_bounds__(inv_plane_threads(M), plane_blocks(M))
         if (2 * pairs <= H) inv_lines<M, true>(src, rs, w, E, Y, SY, l0, nl, 2 * pairs);
         else inv_lines<M, false>(src, rs, w, E, Y, SY, l0, nl, 2 * pairs);
     }
-    // far pairs: this step's node coefficients of field f contracted over z,
-    // then over x (scratch in E)
     const FarTarget *far = I.far;
+    float4 lx[M / 32];                                         // far: x weights of this thread's x < M/2
+    if (far) {
+        const int px = far->px;
+#pragma unroll
+        for (int k2 = 0; k2 < M / 32; ++k2) {
+            const int x = (threadIdx.x & 15) + 16 * k2;
+            const float *l = far->Lx + (x < nx ? x : 0) * px;
+            lx[k2] = make_float4(__ldg(l), px > 1 ? __ldg(l + 1) : 0.0f, px > 2 ? __ldg(l + 2) : 0.0f,
+                                 px > 3 ? __ldg(l + 3) : 0.0f);
+        }
+    }
+    // far pairs: this step's node coefficients of field f contracted over z
+    // (scratch in E), then over y for every row
     if (far) {
         const int px = far->px, py = far->py, pz = far->pz, pxy = px * py;
         const float *c = far->cring + (step % far->depth) * (far->r * 4) + f;
@@ -401,11 +432,12 @@ __global__ void __launch_bounds__(inv_plane_threads(M), plane_blocks(M))
             cz[i] = s;
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < py * nx; i += T) {
-            const int bb = i / nx, x = i - bb * nx;
+        for (int i = threadIdx.x; i < ny * kFarRow; i += T) {
+            const int y = i / kFarRow, a = i % kFarRow;
             float u = 0.0f;
-            for (int aa = 0; aa < px; ++aa) u = fmaf(__ldg(far->Lx + x * px + aa), cz[bb * px + aa], u);
-            ux[i] = u;
+            if (a < px)
+                for (int k = 0; k < py; ++k) u = fmaf(__ldg(far->Ly + y * py + k), cz[k * px + a], u);
+            vy[i] = u;
         }
         __syncthreads();
     }
@@ -415,8 +447,8 @@ __global__ void __launch_bounds__(inv_plane_threads(M), plane_blocks(M))
     constexpr int CP = CH;   // pairs per chunk: 16 B + 1 <= 17 B
     for (int p0 = 0; p0 < pairs; p0 += CP) {
         const int np = min(CP, pairs - p0);
-        if (nx <= H) inv_rows<M, true>(Y, SY, E, tw, p0, np, nx, ny, scale, far, ux, dst);
-        else inv_rows<M, false>(Y, SY, E, tw, p0, np, nx, ny, scale, far, ux, dst);
+        if (nx <= H) inv_rows<M, true>(Y, SY, E, tw, p0, np, nx, ny, scale, far, vy, lx, dst);
+        else inv_rows<M, false>(Y, SY, E, tw, p0, np, nx, ny, scale, far, vy, lx, dst);
     }
 }
 
@@ -432,11 +464,11 @@ size_t smem_fwd_plane_line(int M, int ny)
     return sizeof(float2) * (M + (size_t)((ny + 1) / 2) * 17 * B + (size_t)fwd_chunk(M) * (16 * B + 1));
 }
 
-size_t smem_inv_plane_line(int M, int nx, int ny)
+size_t smem_inv_plane_line(int M, int ny)
 {
     const size_t B = M / 16;
     return sizeof(float2) * (M + (size_t)(M / 2 + 1) * inv_row_stride(M, ny) + (size_t)inv_chunk(M) * 17 * B) +
-           sizeof(float) * (size_t)kMaxFarPts * nx;
+           sizeof(float) * (size_t)kFarRow * ny;
 }
 
 cudaError_t open_plane_line_smem(int max_optin)
