@@ -1,10 +1,11 @@
 // Spectral multiply-accumulate + inverse column FFT, fed by the tensor memory
 // accelerator.
 //
-// For every padded shape with a column class (rp_internal.h).  Same arithmetic as k_mac_inv_column (the sum over a target's (source, lag)
+// For every padded shape with a column class (rp_internal.h).  Same
+// arithmetic as k_mac_inv_column (the sum over a target's (source, lag)
 // entries of G_m * S(l - m), Eq. 12 in the spectral domain, then the inverse
-// FFT along z kept to the target's z < nz), restructured so that the
-// operands stream through shared memory asynchronously:
+// FFT along z kept to the target's z < nz), restructured so that the operands
+// stream through shared memory asynchronously:
 //
 //   * persistent blocks, one per SM, each walking (kx, 16-ky) column tiles
 //     (or two fields or one of a tile, mac_tma_fields);
@@ -138,15 +139,19 @@ __device__ __forceinline__ int owner(const T *arr, int lo, int hi, int b, int T:
     return lo;
 }
 
-// Kahan-compensated addition: s + c carries the sum of the added terms with
-// the rounding of each addition kept in c (the error stays near one rounding
-// of the sum of magnitudes, whatever the number of terms); the total is s - c.
-__device__ __forceinline__ void kahan_add(float &s, float &c, float x)
+// Kahan-compensated addition of two values at a time in packed FP32: s + c
+// carries the sum of the added terms with the rounding of each addition kept
+// in c (the error stays near one rounding of the sum of magnitudes, whatever
+// the number of terms); the total is s - c.  A difference a - b is b * -1 + a,
+// the same one rounding.
+__device__ __forceinline__ void kahan_add2(float &s0, float &s1, float &c0, float &c1, float2 x)
 {
-    const float y = x - c;
-    const float t = s + y;
-    c = (t - s) - y;
-    s = t;
+    const float2 minus = make_float2(-1.0f, -1.0f), s = make_float2(s0, s1), c = make_float2(c0, c1);
+    const float2 y = __ffma2_rn(c, minus, x);
+    const float2 t = __fadd2_rn(s, y);
+    const float2 d = __ffma2_rn(y, minus, __ffma2_rn(s, minus, t));
+    s0 = t.x; s1 = t.y;
+    c0 = d.x; c1 = d.y;
 }
 
 // barrier `id` among the first (or last) `threads` threads of the block
@@ -406,10 +411,8 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
                                 const float4 s = S4[r * 8 + p];
                                 if constexpr (COMP) {
                                     float4 &c = cmp[COMP ? i : 0][f];
-                                    kahan_add(a[i][f].x, c.x, g[i].x * s.x);
-                                    kahan_add(a[i][f].y, c.y, g[i].x * s.y);
-                                    kahan_add(a[i][f].z, c.z, g[i].y * s.z);
-                                    kahan_add(a[i][f].w, c.w, g[i].y * s.w);
+                                    kahan_add2(a[i][f].x, a[i][f].y, c.x, c.y, make_float2(g[i].x * s.x, g[i].x * s.y));
+                                    kahan_add2(a[i][f].z, a[i][f].w, c.z, c.w, make_float2(g[i].y * s.z, g[i].y * s.w));
                                 } else {
                                     a[i][f].x = fmaf(g[i].x, s.x, a[i][f].x);
                                     a[i][f].y = fmaf(g[i].x, s.y, a[i][f].y);
@@ -447,10 +450,10 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
                                 float4 &x = a[i][f];
                                 if constexpr (COMP) {
                                     float4 &c = cmp[COMP ? i : 0][f];
-                                    kahan_add(x.x, c.x, fmaf(g[i].x, s.x, -g[i].y * s.y));
-                                    kahan_add(x.y, c.y, fmaf(g[i].x, s.y, g[i].y * s.x));
-                                    kahan_add(x.z, c.z, fmaf(g[i].z, s.z, -g[i].w * s.w));
-                                    kahan_add(x.w, c.w, fmaf(g[i].z, s.w, g[i].w * s.z));
+                                    kahan_add2(x.x, x.y, c.x, c.y, make_float2(fmaf(g[i].x, s.x, -g[i].y * s.y),
+                                                                               fmaf(g[i].x, s.y, g[i].y * s.x)));
+                                    kahan_add2(x.z, x.w, c.z, c.w, make_float2(fmaf(g[i].z, s.z, -g[i].w * s.w),
+                                                                               fmaf(g[i].z, s.w, g[i].w * s.z)));
                                 } else {
                                     x.x = fmaf(g[i].x, s.x, fmaf(-g[i].y, s.y, x.x));
                                     x.y = fmaf(g[i].x, s.y, fmaf(g[i].y, s.x, x.y));
