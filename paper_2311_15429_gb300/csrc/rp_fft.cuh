@@ -56,7 +56,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // waits for their pipe (32 x 48^3, MAC 380 -> 416 us).
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b)
 {
-#if defined(__CUDA_ARCH__) && !defined(RP_SCALAR_COMPLEX)
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000 && !defined(RP_SCALAR_COMPLEX)
     return __fadd2_rn(a, b);
 #else
     return make_float2(a.x + b.x, a.y + b.y);
@@ -64,7 +64,7 @@ __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b)
 }
 __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b)
 {
-#if defined(__CUDA_ARCH__) && !defined(RP_SCALAR_COMPLEX)
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000 && !defined(RP_SCALAR_COMPLEX)
     return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
 #else
     return make_float2(a.x - b.x, a.y - b.y);
