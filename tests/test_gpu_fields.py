@@ -106,3 +106,35 @@ def test_dipole_field_end_to_end():
     sB = Q * a * math.hypot(omega ** 2 / (c * c * d), omega / (c * d * d))
     assert abs(E[2, k] - Ez) < 3e-3 * sE, (E[2, k], Ez)
     assert abs(B[1, k] - By) < 3e-3 * sB, (B[1, k], By)
+
+
+@pytest.mark.parametrize("n,shift", [((4, 3, 3), 0), ((8, 5, 4), 0), ((64, 6, 5), 0), ((8, 5, 4), 1), ((9, 16, 16), 0),
+                                     ((132, 3, 7), 0)])
+def test_fields_rows_of_four(n, shift):
+    """Rows of whole and broken groups of four nodes, and buffers off a 16-byte
+    boundary: the CUDA stencils against the FP64 oracle's, within FP32 rounding."""
+    import torch
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(4)
+    N = n[0] * n[1] * n[2]
+    phi = rng.standard_normal(N).astype(np.float32)
+    A = [rng.standard_normal(3 * N).astype(np.float32) for _ in range(3)]
+    c, dt, h = synth.C_AU, 0.05, 0.3
+
+    def t(x):
+        buf = torch.zeros(x.size + shift, device=dev)
+        buf[shift:] = torch.from_numpy(x).to(dev)
+        return buf[shift:]
+
+    ctx = rp.rp_create(c, dt, mode=rp.RP_MODE_DIRECT)
+    try:
+        rp.rp_add_domain(ctx, (0.0, 0.0, 0.0), n, h)
+        rp.rp_finalize(ctx)
+        E, B = t(np.zeros(3 * N, np.float32)), t(np.zeros(3 * N, np.float32))
+        rp.rp_fields(ctx, 0, t(phi), t(A[0]), t(A[1]), t(A[2]), E, B)
+        rp.rp_sync(ctx)
+        wantE, wantB = ofields.fields(phi, *[a.reshape(3, N) for a in A], n, h, c, dt)
+        for got, want in ((E, wantE), (B, wantB)):
+            np.testing.assert_allclose(got.cpu().numpy().reshape(3, N), want, rtol=2e-6, atol=2e-6 * np.abs(want).max())
+    finally:
+        rp.rp_destroy(ctx)
