@@ -78,6 +78,7 @@ class RPError(RuntimeError):
 
 
 _lib = None
+_torch_float32 = None
 _V = ctypes.c_void_p
 _I = ctypes.c_int
 _PP = ctypes.POINTER(ctypes.c_void_p)
@@ -153,12 +154,17 @@ def load(build: bool = True):
 
 def _ptr(x) -> int:
     """Raw address of a torch tensor, numpy array or int."""
+    global _torch_float32
     if x is None:
         return 0
     if isinstance(x, int):
         return x
     if hasattr(x, "data_ptr"):
-        if str(x.dtype) != "torch.float32" or not x.is_contiguous():
+        if x.dtype is not _torch_float32:
+            if str(x.dtype) != "torch.float32":
+                raise ValueError("tensor must be contiguous float32")
+            _torch_float32 = x.dtype    # later tensors by identity: the text of a dtype costs a microsecond
+        if not x.is_contiguous():
             raise ValueError("tensor must be contiguous float32")
         return x.data_ptr()
     if hasattr(x, "ctypes"):
@@ -170,10 +176,10 @@ def _ptr(x) -> int:
 
 
 def _ptr_array(xs: Sequence):
-    if isinstance(xs, ctypes.Array):   # made by pointer_array
-        return ctypes.cast(xs, _PP), xs
-    arr = (ctypes.c_void_p * len(xs))(*[_ptr(x) for x in xs])
-    return ctypes.cast(arr, _PP), arr
+    """The argument for a pointer-array parameter (ctypes passes an array as
+    the address of its first element) and what must outlive the call."""
+    arr = xs if isinstance(xs, ctypes.Array) else pointer_array(xs)   # made by pointer_array, or now
+    return arr, arr
 
 
 def pointer_array(xs: Sequence):
