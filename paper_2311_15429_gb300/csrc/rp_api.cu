@@ -147,6 +147,18 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
         const int cls = column_class(g.cls);
         if (cls == 0) continue;
         g.fields = mac_tma_fields(cls, ctx->comp, g.blk1 - g.blk0, ctx->sm_count);
+        // two targets that read the same ring at the same lag; same tiles in all
+        std::map<std::pair<const float2 *, int>, int> reader;
+        bool shared = false, same = true;
+        for (int t = g.i0; t < g.i1; ++t) {
+            const InvTarget &I = ctx->inv[t];
+            same = same && I.kx == ctx->inv[g.i0].kx && I.ay.M == ctx->inv[g.i0].ay.M;
+            for (int e = I.e0; e < I.e1; ++e) {
+                const auto it = reader.emplace(std::make_pair(ctx->entries[e].ring, ctx->entries[e].lag), t);
+                shared = shared || it.first->second != t;
+            }
+        }
+        g.share = shared && same;
         g.stages = mac_tma_stages(cls, max_optin, g.fields);
         if (ctx->cfg.mac_stages >= 2) g.stages = std::min(g.stages, ctx->cfg.mac_stages);
         if (g.stages < 2) {
@@ -741,7 +753,7 @@ rp_status autotune_mac(rp_ctx *ctx)
         float best = 1e30f;
         for (int cw : {8, 12, 16}) {
             auto go = [&] {
-                return launch_mac_tma(cls, cw, false, ctx->d_inv, g.i0, g.i1, g.blk0, ntiles, ctx->d_entries, step, 0,
+                return launch_mac_tma(cls, cw, false, ctx->d_inv, g.i0, g.i1, g.blk0, ntiles, g.share, ctx->d_entries, step, 0,
                                       g.fields, g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
             };
             cudaError_t e = go();
@@ -1243,7 +1255,11 @@ rp_status rp_finalize(rp_ctx *ctx)
             if ((st = dev_alloc(ctx, &ctx->ground[d], n4)) || (st = dev_alloc(ctx, &ctx->delta[d], n4)) ||
                 (st = dev_alloc(ctx, &ctx->pstatic[d], n4)))
                 return st;
+            const GroundDomain *last = ctx->gdom.empty() ? nullptr : &ctx->gdom.back();
+            ctx->gdom.push_back({ctx->ground[d], ctx->delta[d], ctx->doms[d].N,
+                                 last ? last->block0 + ground_blocks(last->n) : 0, 0});
         }
+        if ((st = upload(ctx, &ctx->d_gdom, ctx->gdom))) return st;
     }
     for (InvTarget &I : ctx->inv) {
         if ((st = dev_alloc(ctx, &I.t2, 4ULL * I.kx * I.nz * I.ay.M))) return st;
@@ -1654,6 +1670,7 @@ extern "C" {
 static rp_status split_inputs(rp_ctx *ctx, int d0, int d1, IoPtrs &in)
 {
     if (!ctx->split) return RP_OK;
+    int nblocks = 0;
     for (int d = d0; d < d1; ++d) {
         const long long N = ctx->doms[d].N;
         if (ctx->step == 0) {
@@ -1662,11 +1679,14 @@ static rp_status split_inputs(rp_ctx *ctx, int d0, int d1, IoPtrs &in)
             RP_CUDA(ctx, cudaMemcpyAsync(ctx->ground[d] + N, in.J[d], 3 * N * sizeof(float),
                                          cudaMemcpyDeviceToDevice, ctx->stream));
         } else {
-            RP_CUDA(ctx, launch_ground_delta(in.rho[d], in.J[d], ctx->ground[d], ctx->delta[d], N, ctx->sm_count,
-                                             ctx->stream));
-            in.rho[d] = ctx->delta[d];
-            in.J[d] = ctx->delta[d] + N;
+            nblocks += ground_blocks(N);
         }
+    }
+    if (ctx->step == 0) return RP_OK;
+    RP_CUDA(ctx, launch_ground_delta(ctx->d_gdom, d0, d1, nblocks, in, ctx->stream));
+    for (int d = d0; d < d1; ++d) {
+        in.rho[d] = ctx->delta[d];
+        in.J[d] = ctx->delta[d] + ctx->doms[d].N;
     }
     return RP_OK;
 }
@@ -1901,7 +1921,7 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
         if ((st = timed_launch(ctx, RP_K_MAC_INV_COLUMN, "MAC + inverse column pass", [&] {
                  if (const int cls = column_class(g.cls); ctx->tma && cls > 0)
                      return launch_mac_tma(cls, ctx->mac_cw[class_slot(cls)], ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0,
-                                           ntiles, ctx->d_entries, kstep, clamp, g.fields, g.stages, ctx->sm_count,
+                                           ntiles, g.share, ctx->d_entries, kstep, clamp, g.fields, g.stages, ctx->sm_count,
                                            ctx->d_err, ctx->stream);
                  return launch_mac_inv_column(ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0, ctx->d_entries, ntiles,
                                               ctx->smem_mac, kstep, clamp, ctx->stream);

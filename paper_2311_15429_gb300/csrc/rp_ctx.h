@@ -58,6 +58,7 @@ struct LaunchGroup {
     int blk0, blk1;
     int blk2_0, blk2_1;
     int fields = 0, stages = 0;   // MAC launches: fields of a block's unit, field stages of its pipeline
+    bool share = false;           // MAC launches: targets with the same tiles that read the same source slots
 };
 
 // History spill (RP_FLAG_HISTORY_SPILL).  A source domain with a spilled
@@ -122,6 +123,8 @@ struct rp_ctx {
     cudaGraphExec_t graph_exec = nullptr;
     long long graph_synced = -2;              // host step the device counter holds (-2: unknown)
     std::vector<float *> ground, delta, pstatic;
+    std::vector<GroundDomain> gdom;           // their table for the Delta S launch
+    GroundDomain *d_gdom = nullptr;
     // history spill to host memory (RP_FLAG_HISTORY_SPILL): the spilled
     // sources (host ring depth spill_hd), the windows with their descriptors
     // for the forward passes, and the copy streams with their events:

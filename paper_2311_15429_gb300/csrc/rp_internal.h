@@ -276,14 +276,23 @@ constexpr int kDirMaxLags = 226;   // longest lag window of a direct pair
 
 // Ground-state split and graph-replay step counter (rp_ground.cu).
 cudaError_t launch_step_advance(long long *d_step, cudaStream_t s);
-cudaError_t launch_ground_delta(const float *rho, const float *J, const float *ground, float *delta, long long N,
-                                int sms, cudaStream_t s);
+struct GroundDomain {        // ground-state split: a domain's S(0) and Delta S, [4][n] each
+    const float *ground;
+    float *delta;
+    long long n;
+    int block0;              // its first block in a launch over every domain
+    int pad_;
+};
+int ground_blocks(long long n);
+cudaError_t launch_ground_delta(const GroundDomain *d_doms, int d0, int d1, int nblocks, const IoPtrs &in,
+                                cudaStream_t s);
 
 // Fields from the potentials (rp_fields.cu).
 cudaError_t launch_fields(int nx, int ny, int nz, double h, double c, double dt, const float *phi, const float *A,
                           const float *A1, const float *A2, float *E, float *B, cudaStream_t s);
 
-// TMA-fed MAC (rp_mac_tma.cu): column classes 32..192.
+// TMA-fed MAC (rp_mac_tma.cu): column classes 32..192.  share: the launch's
+// targets have the same tiles and read some of the same source slots.
 int mac_tma_fields(int M, bool comp, int ntiles, int sms);   // fields of a block's unit of work
 int mac_tma_stages(int M, int smem_optin, int fields);
 cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_t s);
@@ -292,8 +301,8 @@ cudaError_t open_mac_tma_smem_limit(int max_optin);
 // comp: the Kahan-compensated variant (consumer_warps must be kCompWarps)
 constexpr int kCompWarps = 12;
 cudaError_t launch_mac_tma(int cls, int consumer_warps, bool comp, const InvTarget *d_tgts, int t0, int t1,
-                           int tile_lo, int ntiles, const MacEntry *d_entries, long long step, int clamp, int fields,
-                           int nstages, int sms, int *d_err, cudaStream_t s);
+                           int tile_lo, int ntiles, bool share, const MacEntry *d_entries, long long step, int clamp,
+                           int fields, int nstages, int sms, int *d_err, cudaStream_t s);
 
 // tcgen05 bf16 GEMM (rp_gemm_tc.cu): D (M x N fp32) = A (M x K) * B (N x K)^T
 bool encode_bf16_rows(void *encode_fn, struct CUtensorMap_st *map, const void *base, uint64_t rows,
