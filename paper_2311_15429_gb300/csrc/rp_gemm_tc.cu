@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "rp_fft.cuh"
 #include "rp_internal.h"
 #include "rp_tc.cuh"
 
@@ -89,6 +90,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    pdl_trigger();
+    pdl_wait();   // the operands, and the last readers of D
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
@@ -247,7 +250,8 @@ bool encode_bf16_rows(void *encode_fn, CUtensorMap *map, const void *base, uint6
 // `splits` > 1 runs split-K: partial products go to `work`
 // (splits x M x N floats) and a reduction writes D (then ldd must be N).
 // `split3`: A and B are [hi | lo] pairs (2K wide) and D is the
-// three-product sum.
+// three-product sum.  `bn`: another column tile (0: the default), a divisor
+// of N and the B map's box rows.
 int gemm_tile_n(int N)
 {
     if (N <= 0 || N % 32) return 0;
@@ -258,10 +262,10 @@ int gemm_tile_n(int N)
 
 cudaError_t launch_gemm_bf16_tn(const CUtensorMap &mapA, const CUtensorMap &mapB, float *D, int M, int N, int K,
                                 int ldd, int smem_optin, int *d_err, cudaStream_t s, int splits, float *work,
-                                int split3, int f16)
+                                int split3, int f16, int bn)
 {
-    const int BNv = gemm_tile_n(N);
-    if (M % kBM || K % kBK || !BNv || splits < 1) return cudaErrorInvalidValue;
+    const int BNv = bn ? bn : gemm_tile_n(N);
+    if (M % kBM || K % kBK || !BNv || N % BNv || splits < 1) return cudaErrorInvalidValue;
     if (splits > 1 && (!work || ldd != N)) return cudaErrorInvalidValue;
     const int kt_all = K / kBK;
     const int kchunk = (kt_all + splits - 1) / splits;
@@ -276,8 +280,8 @@ cudaError_t launch_gemm_bf16_tn(const CUtensorMap &mapA, const CUtensorMap &mapB
     auto go = [&](auto kern, size_t smem, int bn) {
         e = open_smem(kern, smem);
         if (!e)
-            kern<<<grid, kGemmThreads, smem, s>>>(mapA, mapB, out, K, ldd, stages, d_err, kchunk, stride,
-                                                  idesc_16bit(bn, f16));
+            e = launch_pdl(kern, grid, dim3(kGemmThreads), smem, s, mapA, mapB, out, K, ldd, stages, d_err, kchunk,
+                           stride, idesc_16bit(bn, f16));
     };
 #define RP_GEMM_CASE(BN)                                                                             \
     case BN:                                                                                         \

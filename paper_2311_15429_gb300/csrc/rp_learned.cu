@@ -17,6 +17,7 @@
 #include <cstring>
 #include <vector>
 
+#include "rp_fft.cuh"
 #include "rp_learned.h"
 
 namespace rp {
@@ -25,6 +26,13 @@ namespace {
 
 constexpr int kDims[5] = {kLIn, kLHid, kLHid, kLHid, kLOut};
 
+// Column tile of the forward GEMMs: the rows of a step's pairs are a handful
+// of 128-row tiles (8 for 16 domains), so a layer in one 256-column tile runs
+// on as many SMs and its time is the epilogue's; four tiles of 64 take a
+// quarter of it each (9.6 -> 6.1 us a layer).
+constexpr int kFwdCols = 64;
+static_assert(kLHid % kFwdCols == 0 && kLOut % kFwdCols == 0, "whole column tiles");
+
 // ---------------------------------------------------------------- elementwise kernels
 
 // A = leaky(Z) in fp16, and (if At) its transpose; a block is a 32 x 32 tile.
@@ -32,6 +40,9 @@ __global__ void k_act_fwd(const float *__restrict__ Z, __half *__restrict__ A, _
 {
     __shared__ __half t[32][33];
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    pdl_trigger();
+    pdl_wait();
+#pragma unroll 4
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const size_t o = (size_t)(r0 + i) * n + c0 + threadIdx.x;
         const float z = Z[o];
@@ -179,16 +190,20 @@ __global__ void __launch_bounds__(kLinSlices * kLOut) k_linear(const float *__re
     __shared__ float xs[kLinRows][kLIn];
     __shared__ float part[kLinSlices][kLinRows][kLOut];
     const int r0 = blockIdx.x * kLinRows;
-    for (int i = threadIdx.x; i < kLinRows * kLIn; i += blockDim.x) {
-        const int rr = r0 + i / kLIn;
+    pdl_trigger();
+    pdl_wait();
+    static_assert(kLinRows * kLIn % (kLinSlices * kLOut) == 0, "whole rounds");
+#pragma unroll   // every load of a thread in flight
+    for (int k = 0; k < kLinRows * kLIn / (kLinSlices * kLOut); ++k) {
+        const int i = threadIdx.x + k * kLinSlices * kLOut, rr = r0 + i / kLIn;
         xs[i / kLIn][i % kLIn] = rr < rows ? X[(size_t)rr * kLIn + i % kLIn] : 0.0f;
     }
     __syncthreads();
     const int q = threadIdx.x / kLOut, o = threadIdx.x % kLOut;
     constexpr int per = kLIn / kLinSlices;
     float acc[kLinRows] = {};
-#pragma unroll 4
-    for (int i = q * per; i < (q + 1) * per; ++i) {
+#pragma unroll 16
+    for (int i = q * per; i < (q + 1) * per; ++i) {   // the weights' loads, 16 in flight, are what this waits on
         const float w = __ldg(WT + (size_t)i * kLOut + o);
 #pragma unroll
         for (int rr = 0; rr < kLinRows; ++rr) acc[rr] = fmaf(w, xs[rr][i], acc[rr]);
@@ -332,8 +347,7 @@ cudaError_t mlp_create(Mlp &n, int cap, uint64_t seed, void *enc)
         ok = ok && encode_bf16_rows(enc, &n.mA[l], n.A16[l], cap, kLHid, 128) &&
              encode_bf16_rows(enc, &n.mAt[l], n.At16[l], kLHid, cap, (uint32_t)gemm_tile_n(kLHid));
     for (int l = 0; l < 4; ++l) {
-        ok = ok && encode_bf16_rows(enc, &n.mW[l], n.W16[l], kDims[l + 1], kDims[l],
-                                    (uint32_t)gemm_tile_n(kDims[l + 1]));
+        ok = ok && encode_bf16_rows(enc, &n.mW[l], n.W16[l], kDims[l + 1], kDims[l], (uint32_t)kFwdCols);
         if (l > 0)
             ok = ok && encode_bf16_rows(enc, &n.mWt[l], n.Wt16[l], kDims[l], kDims[l + 1],
                                         (uint32_t)gemm_tile_n(kDims[l]));
@@ -406,8 +420,8 @@ cudaError_t linear_apply(const float *Wlin, const float *X, int rows, const floa
                          cudaStream_t s, float scale)
 {
     if (rows <= 0) return cudaSuccess;
-    k_linear<<<(rows + kLinRows - 1) / kLinRows, kLinSlices * kLOut, 0, s>>>(Wlin, X, rows, add, sign, out, scale);
-    return cudaGetLastError();
+    return launch_pdl(k_linear, dim3((rows + kLinRows - 1) / kLinRows), dim3(kLinSlices * kLOut), 0, s, Wlin, X, rows,
+                      add, sign, out, scale);
 }
 
 cudaError_t mlp_zero_last(Mlp &n, cudaStream_t s)
@@ -431,10 +445,13 @@ cudaError_t mlp_forward(Mlp &n, int rows, bool train, int optin, int sms, cudaSt
     cudaError_t e;
     const CUtensorMap *in = &n.mX;
     for (int l = 0; l < 4; ++l) {
-        if ((e = gemm(*in, n.mW[l], n.Z[l], rows, kDims[l + 1], kDims[l], n, optin, sms, s, false))) return e;
+        if ((e = launch_gemm_bf16_tn(*in, n.mW[l], n.Z[l], rows, kDims[l + 1], kDims[l], kDims[l + 1], optin, n.d_err,
+                                     s, 1, nullptr, 0, 1, kFwdCols)))
+            return e;
         if (l < 3) {
-            k_act_fwd<<<dim3(kLHid / 32, rows / 32), dim3(32, 8), 0, s>>>(n.Z[l], n.A16[l], train ? n.At16[l] : nullptr,
-                                                                           kLHid, n.cap);
+            if ((e = launch_pdl(k_act_fwd, dim3(kLHid / 32, rows / 32), dim3(32, 8), 0, s, n.Z[l], n.A16[l],
+                                train ? n.At16[l] : nullptr, kLHid, n.cap)))
+                return e;
             in = &n.mA[l];
         }
     }
