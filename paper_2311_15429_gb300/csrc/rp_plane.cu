@@ -26,7 +26,7 @@
 // skips half of the first layer, cropping (outputs k >= M/2) half of the last.
 //
 // Shared memory per plane of n = M/2 and the blocks an SM holds: M = 96 39 KB
-// (5), M = 128 70 KB (3), M = 192 109 KB (2); the exchange of the y axis goes
+// (5 forward, 4 inverse), M = 128 70 KB (3), M = 192 109 KB (2); the exchange of the y axis goes
 // in chunks of kx lines to keep it there.
 // Per launch, before (tile and lane-shuffle forms) and now: 32 x 48^3 with far
 // pairs forward 111 -> 93 us, inverse 173 -> 117 (288 MB each: 42 us at the
@@ -46,13 +46,16 @@ namespace {
 
 // Threads per block and kx lines per chunk of the y exchange: whole rounds of
 // tasks at n = M/2 (16 and B tasks a line), two chunks at 96 and 128, and at
-// 192 what leaves room for two blocks.
+// 192 what leaves room for two blocks.  The inverse pass at 96 takes four
+// blocks of 208 threads: two rounds a chunk where 160 need three (2 x 48^3
+// 12.6 -> 11.1 us, 32 x 48^3 118 -> 112).
 __host__ __device__ constexpr int plane_threads(int M)
 {
     return M == 32 ? 128 : M == 64 ? 144 : M == 96 ? 160 : M == 128 ? 288 : 320;
 }
-__host__ __device__ constexpr int inv_plane_threads(int M) { return M == 192 ? 224 : plane_threads(M); }
+__host__ __device__ constexpr int inv_plane_threads(int M) { return M == 96 ? 208 : M == 192 ? 224 : plane_threads(M); }
 __host__ __device__ constexpr int plane_blocks(int M) { return M <= 64 ? 6 : M == 96 ? 5 : M == 128 ? 3 : 2; }
+__host__ __device__ constexpr int inv_plane_blocks(int M) { return M == 96 ? 4 : plane_blocks(M); }
 __host__ __device__ constexpr int fwd_chunk(int M) { return M <= 64 ? M / 2 + 1 : M == 96 ? 25 : M == 128 ? 33 : 20; }
 __host__ __device__ constexpr int inv_chunk(int M) { return M <= 64 ? M / 2 + 1 : M == 96 ? 25 : M == 128 ? 33 : 14; }
 // rows y of a kx line between the axes of the inverse pass: even, and B mod 16
@@ -379,7 +382,7 @@ __device__ __forceinline__ void inv_rows(const float2 *Y, int SY, float2 *E, con
 }
 
 template <int M>
-__global__ void __launch_bounds__(inv_plane_threads(M), plane_blocks(M))
+__global__ void __launch_bounds__(inv_plane_threads(M), inv_plane_blocks(M))
     k_inv_plane_line(const InvTarget *__restrict__ tgts, int t0, int t1, int block_lo, OutPtrs out, float inv_c,
                      long long step)
 {
