@@ -159,6 +159,8 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
             }
         }
         g.share = shared && same;
+        g.fft_warps = mac_tma_fft_warps(cls, ctx->comp, g.fields,
+                                        (double)(ctx->inv[g.i1 - 1].e1 - ctx->inv[g.i0].e0) / (g.i1 - g.i0));
         g.stages = mac_tma_stages(cls, max_optin, g.fields);
         if (ctx->cfg.mac_stages >= 2) g.stages = std::min(g.stages, ctx->cfg.mac_stages);
         if (g.stages < 2) {
@@ -754,7 +756,7 @@ rp_status autotune_mac(rp_ctx *ctx)
         for (int cw : {8, 12, 16}) {
             auto go = [&] {
                 return launch_mac_tma(cls, cw, false, ctx->d_inv, g.i0, g.i1, g.blk0, ntiles, g.share, ctx->d_entries, step, 0,
-                                      g.fields, g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
+                                      g.fields, g.fft_warps, g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
             };
             cudaError_t e = go();
             if (!e) e = cudaEventRecord(a, ctx->stream);
@@ -1921,8 +1923,8 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
         if ((st = timed_launch(ctx, RP_K_MAC_INV_COLUMN, "MAC + inverse column pass", [&] {
                  if (const int cls = column_class(g.cls); ctx->tma && cls > 0)
                      return launch_mac_tma(cls, ctx->mac_cw[class_slot(cls)], ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0,
-                                           ntiles, g.share, ctx->d_entries, kstep, clamp, g.fields, g.stages, ctx->sm_count,
-                                           ctx->d_err, ctx->stream);
+                                           ntiles, g.share, ctx->d_entries, kstep, clamp, g.fields, g.fft_warps,
+                                           g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
                  return launch_mac_inv_column(ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0, ctx->d_entries, ntiles,
                                               ctx->smem_mac, kstep, clamp, ctx->stream);
              })))

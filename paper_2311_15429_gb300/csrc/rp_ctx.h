@@ -57,7 +57,8 @@ struct LaunchGroup {
     int i0, i1;
     int blk0, blk1;
     int blk2_0, blk2_1;
-    int fields = 0, stages = 0;   // MAC launches: fields of a block's unit, field stages of its pipeline
+    int fields = 0, stages = 0;   // MAC launches: fields of a block's unit, field stages of its pipeline,
+    int fft_warps = 0;            // warps of its inverse FFT
     bool share = false;           // MAC launches: targets with the same tiles that read the same source slots
 };
 

@@ -294,6 +294,7 @@ cudaError_t launch_fields(int nx, int ny, int nz, double h, double c, double dt,
 // TMA-fed MAC (rp_mac_tma.cu): column classes 32..192.  share: the launch's
 // targets have the same tiles and read some of the same source slots.
 int mac_tma_fields(int M, bool comp, int ntiles, int sms);   // fields of a block's unit of work
+int mac_tma_fft_warps(int M, bool comp, int fields, double entries);
 int mac_tma_stages(int M, int smem_optin, int fields);
 cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_t s);
 size_t mac_tma_smem(int M, int nstages, int fields);
@@ -302,7 +303,7 @@ cudaError_t open_mac_tma_smem_limit(int max_optin);
 constexpr int kCompWarps = 12;
 cudaError_t launch_mac_tma(int cls, int consumer_warps, bool comp, const InvTarget *d_tgts, int t0, int t1,
                            int tile_lo, int ntiles, bool share, const MacEntry *d_entries, long long step, int clamp,
-                           int fields, int nstages, int sms, int *d_err, cudaStream_t s);
+                           int fields, int fft_warps, int nstages, int sms, int *d_err, cudaStream_t s);
 
 // tcgen05 bf16 GEMM (rp_gemm_tc.cu): D (M x N fp32) = A (M x K) * B (N x K)^T
 bool encode_bf16_rows(void *encode_fn, struct CUtensorMap_st *map, const void *base, uint64_t rows,

@@ -196,10 +196,17 @@ __device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw,
     }
 }
 
-// Warps of the inverse column FFT: fewer in the compensated variant, whose
-// MAC warps hold twice the accumulators and need the registers.
-template <bool COMP>
-__host__ __device__ constexpr int fft_warps() { return COMP ? 3 : kFftWarps; }
+// Warps of the inverse column FFT (FW): seven beside the plain sum's MAC
+// warps; beside the compensated ones, whose accumulators need the registers,
+// three, which keep up with tiles of many entries and leave the multiply-adds
+// the issue slots.  Tiles of few entries (the self lags alone) wait for them:
+// there as many as the registers leave, seven up to M = 64 and five at 96 (at
+// 128 and 192 none are left).  32 x 48^3, 4 entries a tile: MAC 382 us with
+// three, 354 with five; 2 x 48^3, 9 entries: 52.6 and 54.4; 64^3 class of the
+// mixed sizes, 4 entries: 27.3 with three, 25.9 with seven; four 27^3
+// neighbours, 19 entries: 62.2 and 66.1.
+constexpr int kFewEntries = 6;
+__host__ __device__ constexpr int few_fft_warps(int M) { return M <= 64 ? 7 : M == 96 ? 5 : 3; }
 
 // A block's unit of work is FH fields of one tile: all four (the kernel tile
 // read once), unless
@@ -218,12 +225,12 @@ __host__ __device__ constexpr int fft_warps() { return COMP ? 3 : kFftWarps; }
 // entries of 4.3 MB over 155 MB of distinct slots: 93.4 -> 85.3 us per step.
 
 // M: padded FFT size along z; CW: multiply-accumulate warps (the block has
-// CW + fft_warps + 1); FPC: field tiles per ring copy (1, 2 or 4; they are
+// CW + FW + 1); FPC: field tiles per ring copy (1, 2 or 4; they are
 // contiguous in the ring); FH: fields of a unit; COMP: the sum over (source,
 // lag) entries is Kahan-compensated per spectral coefficient (the default;
 // RP_FLAG_PLAIN_SUM selects the plain chain).
-template <int M, int CW, int FPC, int FH, bool COMP>
-__global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
+template <int M, int CW, int FPC, int FH, int FW, bool COMP>
+__global__ void __launch_bounds__((CW + FW + 1) * 32, 1)
     k_mac_tma(const InvTarget *__restrict__ tgts, int t0, int t1, int tile_lo, int nunits, int share,
               const MacEntry *__restrict__ entries, long long step, int clamp, int ns, int *err)
 {
@@ -231,7 +238,6 @@ __global__ void __launch_bounds__((CW + fft_warps<COMP>() + 1) * 32, 1)
     constexpr int SSTAGE = FPC * STAGE;             // FPC field tiles of one entry
     constexpr int NG = kKernelStages;
     constexpr int kConsumerWarps = CW;
-    constexpr int FW = fft_warps<COMP>();
     constexpr int RSTEP = kConsumerWarps * 32 / 8;   // rows covered by one pass of the consumers
     constexpr int ROWS = (M + RSTEP - 1) / RSTEP;
     constexpr int FS = M * kTileY;                   // float2 per field of the FFT tile (dense rows)
@@ -535,14 +541,19 @@ constexpr int fields_per_copy(int M, int fh)
 constexpr bool unit_runs(int M, int fh, bool comp) { return !(comp && M == 192 && fh == 4); }
 
 template <int M, int FH, class F>
-cudaError_t for_variants(F &&f)   // f(kernel, consumer warps, compensated)
+cudaError_t for_variants(F &&f)   // f(kernel, multiply-add warps, FFT warps, compensated)
 {
     constexpr int FPC = fields_per_copy(M, FH);
     cudaError_t e;
-    if ((e = f(k_mac_tma<M, 8, FPC, FH, false>, 8, false)) || (e = f(k_mac_tma<M, 12, FPC, FH, false>, 12, false)) ||
-        (e = f(k_mac_tma<M, 16, FPC, FH, false>, 16, false)))
+    constexpr int FW = kFftWarps, FEW = few_fft_warps(M);
+    if ((e = f(k_mac_tma<M, 8, FPC, FH, FW, false>, 8, FW, false)) ||
+        (e = f(k_mac_tma<M, 12, FPC, FH, FW, false>, 12, FW, false)) ||
+        (e = f(k_mac_tma<M, 16, FPC, FH, FW, false>, 16, FW, false)))
         return e;
-    if constexpr (unit_runs(M, FH, true)) return f(k_mac_tma<M, kCompWarps, FPC, FH, true>, kCompWarps, true);
+    if constexpr (unit_runs(M, FH, true)) {
+        if ((e = f(k_mac_tma<M, kCompWarps, FPC, FH, 3, true>, kCompWarps, 3, true))) return e;
+        if constexpr (FEW != 3 && FH == 4) return f(k_mac_tma<M, kCompWarps, FPC, FH, FEW, true>, kCompWarps, FEW, true);
+    }
     return cudaSuccess;
 }
 
@@ -568,6 +579,13 @@ int mac_tma_fields(int M, bool comp, int ntiles, int sms)
     return fh;
 }
 
+// FFT warps of a launch whose targets have `entries` (source, lag) terms on average.
+int mac_tma_fft_warps(int M, bool comp, int fh, double entries)
+{
+    if (!comp) return kFftWarps;
+    return fh == 4 && entries <= kFewEntries ? few_fft_warps(M) : 3;
+}
+
 int mac_tma_stages(int M, int smem_optin, int fh)
 {
     const long long sstage = (long long)fields_per_copy(M, fh) * M * 128;
@@ -587,7 +605,7 @@ size_t mac_tma_smem(int M, int nstages, int fh)
 cudaError_t open_mac_tma_smem_limit(int max_optin)
 {
     cudaError_t e;
-    const auto open = [&](auto kern, int, bool) {
+    const auto open = [&](auto kern, int, int, bool) {
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
     };
 #define X(M, FH) \
@@ -600,7 +618,7 @@ cudaError_t open_mac_tma_smem_limit(int max_optin)
 }
 
 cudaError_t launch_mac_tma(int cls, int cw, bool comp, const InvTarget *d_tgts, int t0, int t1, int tile_lo,
-                           int ntiles, bool share, const MacEntry *d_entries, long long step, int clamp, int fh,
+                           int ntiles, bool share, const MacEntry *d_entries, long long step, int clamp, int fh, int fw,
                            int nstages, int sms, int *d_err, cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
@@ -608,11 +626,11 @@ cudaError_t launch_mac_tma(int cls, int cw, bool comp, const InvTarget *d_tgts, 
     if (nstages < 2 || nstages > kMaxStages || (fh != 4 && fh != 2 && fh != 1) || !unit_runs(cls, fh, comp))
         return cudaErrorInvalidValue;
     const size_t smem = mac_tma_smem(cls, nstages, fh);
-    const int threads = (cw + (comp ? fft_warps<true>() : fft_warps<false>()) + 1) * 32;
+    const int threads = (cw + fw + 1) * 32;
     const int nunits = ntiles * (4 / fh), grid = nunits < sms ? nunits : sms;
     cudaError_t e = cudaErrorInvalidValue;
-    const auto go = [&](auto kern, int w, bool c) {
-        if (w == cw && c == comp)
+    const auto go = [&](auto kern, int w, int f, bool c) {
+        if (w == cw && f == fw && c == comp)
             e = launch_pdl(kern, dim3(grid), dim3(threads), smem, s, d_tgts, t0, t1, tile_lo, nunits, share ? 1 : 0,
                            d_entries, step, clamp, nstages, d_err);
         return cudaSuccess;
