@@ -137,9 +137,9 @@ typedef enum {
 /* By default the spectral sum over a target's (source, lag) entries (Eq. 12
  * per spectral coefficient, before the one inverse FFT per target and field)
  * is Kahan-compensated in FP32: its rounding stays near one rounding of the
- * sum of magnitudes however many entries a target has (the MAC then runs one
- * variant, 12 multiply-add warps and 3 inverse-FFT warps; rp_config.mac_warps
- * must be 0 or 12).  This flag makes it a plain FP32 multiply-add chain,
+ * sum of magnitudes however many entries a target has (the MAC then runs 12
+ * multiply-add warps, with 3 inverse-FFT warps or up to 7 for targets of few
+ * entries; rp_config.mac_warps must be 0 or 12).  This flag makes it a plain FP32 multiply-add chain,
  * whose error grows like the square root of the entry count, with the
  * autotuned 8/12/16-warp variants. */
 #define RP_FLAG_PLAIN_SUM 0x80u
@@ -226,7 +226,7 @@ typedef struct {
                                * window rings, their input slices and the staging rings) */
     long long kernel_bytes;   /* of which: kernel spectra */
     long long points;         /* sum of grid points over all domains */
-    int mac_tma;              /* 1: the spectral MAC of cubic targets is fed by TMA copies */
+    int mac_tma;              /* 1: the spectral MAC of targets with a compiled length along z is fed by TMA copies */
     int npairs_far;           /* pairs on the low-rank far path */
     long long far_bytes;      /* device memory of the far path (factors, batches, rings) */
     int mac_warps;            /* consumer warps of the MAC variant in use (last size class), 0 if none */

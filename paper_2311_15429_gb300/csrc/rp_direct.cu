@@ -26,7 +26,7 @@
 //     its neighbours', on its own).
 // 32^3 (h 0.25) and 27^3 (h 0.3), both cross pairs, 1.29e9 node pairs a step:
 // 7060 us with one thread per target, scalar samples and a Kahan addition per
-// term; 2300 us with two targets per thread and a sample pair each; 1730 us in
+// term; 2300 us with two targets per thread and a sample pair each; 1720 us in
 // this form (55 % of issue slots; neither more warps nor scalar arithmetic in
 // place of the packed changes that).
 #include <cuda_runtime.h>
@@ -128,8 +128,9 @@ __device__ __forceinline__ void direct_run(const float4 *__restrict__ S, const f
                 if (own[i] == jj) inv[i] = tau[i] = 0.0f;
         }
         if constexpr (SHARED) {
-            // the earliest of the four lag intervals and the one after it:
-            // x0 + min(u, 1) (x1 - x0) + max(u - 1, 0) (x2 - x1), u = tau - m
+            // the earliest of the four lag intervals, or the one after it; a
+            // sample outside a target's own interval does not enter its sum
+            // (it may not be finite)
             const float t = __fadd_rd(fminf(fminf(tau[0], tau[1]), fminf(tau[2], tau[3])), kFloorShift);
             const float m0 = t - kFloorShift, m1 = m0 + 1.0f;
             const float4 *s = S + min(__float_as_uint(t) - base, top) * (unsigned)(tile + 1) + jj;
@@ -138,9 +139,16 @@ __device__ __forceinline__ void direct_run(const float4 *__restrict__ S, const f
             const float2 ea = __ffma2_rn(lo2(x1), minus, lo2(x2)), eb = __ffma2_rn(hi2(x1), minus, hi2(x2));
 #pragma unroll
             for (int i = 0; i < kDirOwn; ++i) {
-                const float2 w = dup(__saturatef(tau[i] - m0)), e = dup(__saturatef(tau[i] - m1));
-                acc[i][0] = __ffma2_rn(dup(inv[i]), __ffma2_rn(e, ea, __ffma2_rn(w, da, lo2(x0))), acc[i][0]);
-                acc[i][1] = __ffma2_rn(dup(inv[i]), __ffma2_rn(e, eb, __ffma2_rn(w, db, hi2(x0))), acc[i][1]);
+                const float2 w = dup(tau[i] - m0);
+                float2 va = __ffma2_rn(w, da, lo2(x0)), vb = __ffma2_rn(w, db, hi2(x0));
+                if (tau[i] >= m1) {
+                    const float2 e = dup(tau[i] - m1);
+                    va = __ffma2_rn(e, ea, lo2(x1));
+                    vb = __ffma2_rn(e, eb, hi2(x1));
+                }
+                if (SELF && own[i] == jj) va = vb = dup(0.0f);
+                acc[i][0] = __ffma2_rn(dup(inv[i]), va, acc[i][0]);
+                acc[i][1] = __ffma2_rn(dup(inv[i]), vb, acc[i][1]);
             }
         } else {
 #pragma unroll
@@ -149,9 +157,11 @@ __device__ __forceinline__ void direct_run(const float4 *__restrict__ S, const f
                 const float2 w = dup(tau[i] - (t - kFloorShift));
                 const float4 *s = S + min(__float_as_uint(t) - base, top) * (unsigned)(tile + 1) + jj;
                 const float4 x0 = s[0], x1 = s[tile + 1];
-                const float2 da = __ffma2_rn(lo2(x0), minus, lo2(x1)), db = __ffma2_rn(hi2(x0), minus, hi2(x1));
-                acc[i][0] = __ffma2_rn(dup(inv[i]), __ffma2_rn(w, da, lo2(x0)), acc[i][0]);
-                acc[i][1] = __ffma2_rn(dup(inv[i]), __ffma2_rn(w, db, hi2(x0)), acc[i][1]);
+                float2 va = __ffma2_rn(w, __ffma2_rn(lo2(x0), minus, lo2(x1)), lo2(x0));
+                float2 vb = __ffma2_rn(w, __ffma2_rn(hi2(x0), minus, hi2(x1)), hi2(x0));
+                if (SELF && own[i] == jj) va = vb = dup(0.0f);
+                acc[i][0] = __ffma2_rn(dup(inv[i]), va, acc[i][0]);
+                acc[i][1] = __ffma2_rn(dup(inv[i]), vb, acc[i][1]);
             }
         }
     }

@@ -42,3 +42,32 @@ def test_direct_sum_against_oracle(name):
         want = oracle_values(doms, hists, 0, c, dt, t, T - 1, np.arange(d.N))
         errs = rel_l2(res[T - 1][t], want)
         assert max(errs) <= TOL_BASE + TOL_PER_LAG * lag, (name, t, lag, errs)
+
+
+@pytest.mark.parametrize("mode", [rp.RP_MODE_FFT, rp.RP_MODE_DIRECT])
+def test_direct_sum_reads_each_targets_own_samples(mode):
+    """One sample that is not finite reaches exactly the nodes whose lag
+    interval holds it (neighbours that share a thread's samples do not)."""
+    import torch
+    dev = torch.device("cuda", 0)
+    c, dt = 20.0, 0.05                                     # one light step per bohr
+    doms = [synth.Domain((0.0, 0.0, 0.0), (12, 4, 3), 0.3), synth.Domain((5.0, 0.2, -0.1), (9, 3, 2), 0.25)]
+    with rp.RetardedPotentials(doms, c, dt, mode=mode, flags=rp.RP_FLAG_PLAN_ONLY) as plan:
+        T = plan.query()["max_lag"] + 3
+    rng = np.random.default_rng(11)
+    hists = [rng.standard_normal((T, 4, d.N)).astype(np.float32) for d in doms]
+    bad, lag = 13, 3                                       # a node of domain 1, this many steps back
+    hists[1][T - 1 - lag, 0, bad] = np.inf
+    with rp.RetardedPotentials(doms, c, dt, mode=mode) as lib:
+        for i in range(T):
+            x = [torch.from_numpy(h[i]).to(dev) for h in hists]
+            lib.push_all([v[0].contiguous() for v in x], [v[1:].contiguous().reshape(-1) for v in x])
+        phi, _ = lib.evaluate()
+        got = ~np.isfinite(phi[0].cpu().numpy())
+    src = np.array([v[bad] for v in doms[1].coords()])
+    tau = np.sqrt(sum((a - b) ** 2 for a, b in zip(doms[0].coords(), src))) / (c * dt)
+    assert np.all(np.abs(tau - np.round(tau)) > 1e-4)      # no node on an interval's edge
+    m = np.floor(tau).astype(int)
+    want = (m == lag) | (m == lag - 1)
+    assert want.any() and (~want).any()
+    np.testing.assert_array_equal(got, want)
