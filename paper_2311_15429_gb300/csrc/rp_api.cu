@@ -1156,8 +1156,10 @@ rp_status rp_finalize(rp_ctx *ctx)
             P.nx_s = S.n[0]; P.ny_s = S.n[1]; P.nz_s = S.n[2];
             P.n_s = S.N;
             P.dx = T.o[0] - S.o[0]; P.dy = T.o[1] - S.o[1]; P.dz = T.o[2] - S.o[2];
-            P.hs = S.h;
-            P.vol = (float)(S.h * S.h * S.h);
+            P.scale = std::ldexp(1.0, -std::ilogb(S.h));
+            P.hs = (float)(S.h * P.scale);
+            P.vol = (float)(S.h * S.h * S.h * P.scale);
+            P.inv_cdt = (float)(1.0 / (cdt * P.scale));
             P.is_self = t == s;
             P.self_w = t == s ? (float)(cube_average_constant() * S.h * S.h) : 0.0f;
             P.lag_lo = p.lag_lo;
@@ -1290,7 +1292,7 @@ rp_status rp_finalize(rp_ctx *ctx)
         for (const DirectTarget &D : ctx->dtg) nodes += D.n;
         ctx->dir_splits = ctx->cfg.device_budget > 0 ? 1 : direct_splits(ctx->dir_blocks, least);
         if (ctx->dir_splits > 1) {
-            st = dev_alloc(ctx, &ctx->dir_part, (size_t)(4 * nodes * ctx->dir_splits));
+            st = dev_alloc(ctx, &ctx->dir_part, (size_t)(8 * nodes * ctx->dir_splits));
             if (st == RP_ERR_OOM) {
                 cudaGetLastError();
                 ctx->dir_splits = 1;
@@ -1302,7 +1304,7 @@ rp_status rp_finalize(rp_ctx *ctx)
             long long at = 0;
             for (DirectTarget &D : ctx->dtg) {
                 D.part0 = at;
-                at += 4 * D.n * ctx->dir_splits;
+                at += 8 * D.n * ctx->dir_splits;
             }
         }
     }
@@ -1956,11 +1958,9 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
             return st;
     }
     if (!ctx->dtg.empty()) {
-        const double inv_cdt = 1.0 / (ctx->cfg.c * ctx->cfg.dt);
         if ((st = timed_launch(ctx, RP_K_DIRECT, "direct sum", [&] {
                  return launch_direct(ctx->d_dtg, (int)ctx->dtg.size(), ctx->d_dpairs, out, ctx->dir_part,
-                                      ctx->dir_splits, ctx->dir_blocks, ctx->dir_nlag, kstep, clamp, inv_cdt, inv_c,
-                                      ctx->stream);
+                                      ctx->dir_splits, ctx->dir_blocks, ctx->dir_nlag, kstep, clamp, inv_c, ctx->stream);
              })))
             return st;
     }

@@ -92,8 +92,12 @@ struct DirectPair {
     int nx_s, ny_s, nz_s;
     long long n_s;
     double dx, dy, dz;       // o_t - o_s
-    double hs;
-    float vol;               // hs^3
+    // Lengths in the direct sum are in units of a power of two near the source's
+    // spacing (the bits of a length in bohr, without its underflow)
+    double scale;            // that unit's inverse
+    float hs;                // hs scale
+    float vol;               // hs^3 scale
+    float inv_cdt;           // 1 / (c dt scale)
     float self_w;            // C hs^2 (self pair only)
     int is_self;
     int lag_lo, nlag;        // samples of lags lag_lo .. lag_lo + nlag - 1
@@ -112,7 +116,7 @@ struct DirectTarget {
     int block0;              // first block in the direct grid
     int accumulate;          // add onto the output (FFT pairs wrote it) instead of writing
     int groups, shared;      // groups of four nodes per row (0: consecutive nodes); they share samples
-    long long part0;         // its parts' first float in the workspace ([split][4][n])
+    long long part0;         // its parts' first float in the workspace ([split][4][hi, lo][n])
     const long long *d_step; // the step, for launches made with step < 0 (graph replay)
 };
 
@@ -267,7 +271,7 @@ cudaError_t launch_inv_plane_line(int M, const InvTarget *d_tgts, int t0, int t1
 // part: the workspace of nsplit parts of the sources per target (unused for one)
 cudaError_t launch_direct(const DirectTarget *d_tgts, int ntgt, const DirectPair *d_pairs,
                           const OutPtrs &out, float *part, int nsplit, int nblocks, int max_nlag, long long step,
-                          int clamp, double inv_cdt, float inv_c, cudaStream_t s);
+                          int clamp, float inv_c, cudaStream_t s);
 int direct_groups(int nx, double h, double cdt, bool *shared);
 int direct_blocks(const int n[3], int groups);
 int direct_splits(int blocks, long long min_sources);
