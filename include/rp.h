@@ -188,7 +188,9 @@ typedef struct {
     long long device_budget; /* largest device memory the context may hold, in bytes (rp_stats.device_bytes);
                           * an allocation that would pass it returns RP_ERR_OOM without calling the
                           * allocator (with RP_FLAG_PLAN_ONLY, rp_finalize compares the planned bytes).
-                          * 0: no limit.  Not in the paper: a resource guard of the library. */
+                          * 0: no limit.  Under a limit the direct sums run without the workspace of their
+                          * parts: the same bits from fewer blocks.  Not in the paper: a resource guard of
+                          * the library. */
     int mac_stages;      /* field-tile stages of the TMA-fed MAC's copy pipeline, 2 .. (as many as the
                           * shared memory holds), or 0 for the most that fit; fewer stages leave
                           * shared memory on each SM for other kernels' blocks (the overlapped push's

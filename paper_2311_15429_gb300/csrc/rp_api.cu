@@ -732,6 +732,40 @@ rp_status build_learned(rp_ctx *ctx, const std::vector<float> &weights, const st
     return RP_OK;
 }
 
+// The direct sums' blocks, and the workspace of the targets whose sources run
+// in parts beside one another.  Without it (under a device budget, whose
+// planned bytes it would pass, or where the device has no room) a block runs
+// its targets' parts in turn: the same bits, only fewer blocks.  After every
+// other allocation of the plan.
+rp_status plan_direct(rp_ctx *ctx)
+{
+    long long floats = 0;
+    for (DirectTarget &D : ctx->dtg) {
+        D.part0 = floats;
+        if (D.parts > 1) floats += 8 * D.n * D.parts;
+    }
+    if (floats && ctx->cfg.device_budget <= 0) {
+        const std::string before = ctx->last_error;
+        const rp_status st = dev_alloc(ctx, &ctx->dir_part, (size_t)floats);
+        if (st == RP_ERR_OOM) {
+            cudaGetLastError();
+            ctx->last_error = before;
+        } else if (st) {
+            return st;
+        }
+    }
+    ctx->dir_turn = floats && !ctx->dir_part;
+    ctx->dir_blocks = ctx->dir_sum_blocks = 0;
+    for (DirectTarget &D : ctx->dtg) {
+        const bool beside = !ctx->dir_turn && D.parts > 1;
+        D.block0 = ctx->dir_blocks;
+        D.sum0 = ctx->dir_sum_blocks;
+        ctx->dir_blocks += D.blocks * (beside ? D.parts : 1);
+        ctx->dir_sum_blocks += beside ? D.blocks : 0;
+    }
+    return RP_OK;
+}
+
 // Launch-shape autotuning: time each consumer-warp variant of the TMA-fed MAC
 // on this plan (two launches after one warm-up, on the context stream, over
 // rings whose contents do not matter for timing) and keep the fastest per
@@ -1166,16 +1200,17 @@ rp_status rp_finalize(rp_ctx *ctx)
             P.nlag = p.lag_hi - p.lag_lo + 1;
             max_nlag = std::max(max_nlag, P.nlag);
             rdepth[s] = std::max(rdepth[s], p.lag_hi + 1 + (ctx->overlap ? 1 : 0));
+            D.sources += S.N;
             ctx->dpairs.push_back(P);
         }
         D.p1 = (int)ctx->dpairs.size();
         if (D.p1 > D.p0) {
-            D.block0 = ctx->dir_blocks;
             D.accumulate = tgt_fft[t];
             bool shared = false;
             D.groups = direct_groups(T.n[0], T.h, cdt, &shared);
             D.shared = shared ? 1 : 0;
-            ctx->dir_blocks += direct_blocks(T.n, D.groups);
+            D.blocks = direct_blocks(T.n, D.groups);
+            D.parts = direct_parts(D.blocks, D.sources);
             ctx->dtg.push_back(D);
         }
     }
@@ -1283,31 +1318,6 @@ rp_status rp_finalize(rp_ctx *ctx)
         P.raw = ctx->raw[P.src].ring;
         P.depth = ctx->raw[P.src].depth;
     }
-    if (!ctx->dtg.empty()) {
-        // the direct sums' sources in parts, summed afterwards from a workspace;
-        // in one part, with no workspace, under a device budget or where the
-        // device has no room for it
-        long long least = 0, nodes = 0;
-        for (const DirectPair &P : ctx->dpairs) least = least ? std::min(least, P.n_s) : P.n_s;
-        for (const DirectTarget &D : ctx->dtg) nodes += D.n;
-        ctx->dir_splits = ctx->cfg.device_budget > 0 ? 1 : direct_splits(ctx->dir_blocks, least);
-        if (ctx->dir_splits > 1) {
-            st = dev_alloc(ctx, &ctx->dir_part, (size_t)(8 * nodes * ctx->dir_splits));
-            if (st == RP_ERR_OOM) {
-                cudaGetLastError();
-                ctx->dir_splits = 1;
-            } else if (st) {
-                return st;
-            }
-        }
-        if (ctx->dir_splits > 1) {
-            long long at = 0;
-            for (DirectTarget &D : ctx->dtg) {
-                D.part0 = at;
-                at += 8 * D.n * ctx->dir_splits;
-            }
-        }
-    }
 
     // ---- kernel spectra (FP64 on the host, stored FP32), built in parallel;
     // each target's real and complex kernels are contiguous
@@ -1395,6 +1405,7 @@ rp_status rp_finalize(rp_ctx *ctx)
     if ((st = build_mix(ctx))) return st;
     if ((st = upload(ctx, &ctx->d_inv, ctx->inv))) return st;
     if ((st = upload(ctx, &ctx->d_entries, ctx->entries))) return st;
+    if ((st = plan_direct(ctx))) return st;
     if ((st = upload(ctx, &ctx->d_dtg, ctx->dtg))) return st;
     if ((st = upload(ctx, &ctx->d_dpairs, ctx->dpairs))) return st;
     if ((st = upload(ctx, &ctx->d_raw, ctx->raw))) return st;
@@ -1960,7 +1971,8 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
     if (!ctx->dtg.empty()) {
         if ((st = timed_launch(ctx, RP_K_DIRECT, "direct sum", [&] {
                  return launch_direct(ctx->d_dtg, (int)ctx->dtg.size(), ctx->d_dpairs, out, ctx->dir_part,
-                                      ctx->dir_splits, ctx->dir_blocks, ctx->dir_nlag, kstep, clamp, inv_c, ctx->stream);
+                                      ctx->dir_turn, ctx->dir_blocks, ctx->dir_sum_blocks, ctx->dir_nlag, kstep, clamp, inv_c,
+                                      ctx->stream);
              })))
             return st;
     }

@@ -168,8 +168,9 @@ struct rp_ctx {
     std::vector<int> raw_block0;                     // [ndom + 1], blocks of k_ring_push
     int plane_blocks = 0, col_blocks = 0, mac_blocks = 0, invp_blocks = 0, dir_blocks = 0;
     size_t smem_plane = 0, smem_col = 0, smem_mac = 0, smem_inv = 0;
-    int dir_nlag = 0, dir_splits = 1;                // direct sums: longest lag window, parts of the sources
-    float *dir_part = nullptr;                       // their workspace (more than one part)
+    int dir_nlag = 0, dir_sum_blocks = 0;            // direct sums: longest lag window, blocks that add the parts
+    float *dir_part = nullptr;                       // their workspace (a target with more than one part)
+    bool dir_turn = false;                           // no workspace though a target has: parts in turn
     size_t smem_plane_cls[7] = {}, smem_inv_cls[7] = {}; // plane passes' shared memory per launch (by class_slot)
     int max_lag = 0, raw_depth = 0, spec_depth = 0;
     long long spectral_bytes = 0, kernel_bytes = 0, device_bytes = 0;

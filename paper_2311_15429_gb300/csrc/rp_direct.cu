@@ -19,19 +19,22 @@
 //     they are farther apart, or rows so short that groups of four would be
 //     mostly padding, each target loads its own two (direct_groups);
 //   * the eight warps of a block share 128 targets and divide a staged tile of
-//     sources, and blockIdx.y divides the sources again (direct_splits), so
-//     that small grids fill the chip too; k_direct_sum adds the parts in order;
+//     sources, and the sources run in parts in blocks beside one another
+//     (direct_parts), so that small grids fill the chip too; k_direct_sum adds
+//     the parts in order;
 //   * every term's product and addition is compensated (direct_add), as are
 //     the additions of the warps' and the parts' sums;
 //   * lengths are in bohr but for a power of two (DirectPair::scale), so that
 //     positions on a dyadic grid and their differences stay exact, and no
 //     square of a distance underflows whatever c dt is.  (In units of c dt,
 //     with runs of 8 terms in plain FP32, the sum took 1713 us in place of
-//     1915, at 2 to 5 times the error on white noise at h = 0.25, and NaN from
+//     1870, at 2 to 5 times the error on white noise at h = 0.25, and NaN from
 //     c dt = 1e19 bohr on.)
 // 32^3 (h 0.25) and 27^3 (h 0.3), both cross pairs, 1.29e9 node pairs a step:
 // 6990 us with one thread per target, scalar samples and a Kahan addition per
-// term; 1915 us in this form.
+// term; 1870 us in this form.  One small target under a large source, 9^3 and
+// 36^3: 1525 us with the sources of every target in as many parts as the
+// smallest source allows, 237 with parts by target.
 #include <cuda_runtime.h>
 
 #include "rp_internal.h"
@@ -210,9 +213,11 @@ __device__ __forceinline__ void direct_store(const DirectTarget &T, const OutPtr
     *o = v;
 }
 
-// blockIdx.x: 128 target places (DirectTarget::block0), blockIdx.y: part of
-// the sources.  part: [T.part0 + ((split * 4 + f) * 2 + {hi, lo}) * n + k] when
-// gridDim.y > 1.
+// A block: 128 target places and one part of the target's sources (its pairs'
+// one after another), or (TURN: no workspace) every part in turn, the same
+// sums added in the same order.  part, of targets with more than one:
+// [T.part0 + ((part * 4 + f) * 2 + {hi, lo}) * n + k].
+template <bool TURN>
 __global__ void __launch_bounds__(kDirThreads, 2)
     k_direct(const DirectTarget *__restrict__ tgts, int ntgt, const DirectPair *__restrict__ pairs, OutPtrs out,
              float *__restrict__ part, int tile, int max_nlag, long long step, int clamp, float inv_c)
@@ -231,15 +236,19 @@ __global__ void __launch_bounds__(kDirThreads, 2)
     if (step < 0) step = *T.d_step;   // graph replay: the step from the device counter
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int share = tile / kDirWarps;   // sources of a warp in a full tile
-    const int b = (int)blockIdx.x - T.block0, split = blockIdx.y, nsplit = gridDim.y;
+    const int local = (int)blockIdx.x - T.block0, split0 = TURN ? 0 : local / T.blocks, b = local - split0 * T.blocks;
+    float tot[kDirOut] = {}, err[kDirOut] = {};
 
-    {
+    for (int split = split0; split < (TURN ? T.parts : split0 + 1); ++split) {
         DirectSums sum;
 #pragma unroll
         for (int i = 0; i < kDirOwn; ++i) sum.hi[i][0] = sum.hi[i][1] = sum.lo[i][0] = sum.lo[i][1] = dup(0.0f);
-        for (int p = T.p0; p < T.p1; ++p) {
+        long long before = 0;   // sources of the pairs before
+        for (int p = T.p0; p < T.p1; before += pairs[p].n_s, ++p) {
             const DirectPair &P = pairs[p];
-            const long long j_first = P.n_s * split / nsplit, j_end = P.n_s * (split + 1) / nsplit;
+            const long long j_first = max(T.sources * split / T.parts - before, 0LL);
+            const long long j_end = min(T.sources * (split + 1) / T.parts - before, P.n_s);
+            if (j_first >= j_end) continue;
             const int rows = P.nlag + 3;
             DirectNodes r;   // once in FP64
             {
@@ -264,7 +273,7 @@ __global__ void __launch_bounds__(kDirThreads, 2)
             }
             // low bits of floor(tau) + 2^23, less the lag of sample row 0
             const unsigned base = __float_as_uint(kFloorShift) + (unsigned)(P.lag_lo - 1), top = (unsigned)P.nlag;
-            __syncthreads();   // the rows of the pair before are read
+            __syncthreads();   // the rows of the pair before, or the sums of the part before, are read
             for (int i = threadIdx.x; i < rows; i += kDirThreads) {
                 long long j = step - (P.lag_lo + max(0, min(i - 1, P.nlag - 1)));
                 if (clamp && j < 0) j = 0;
@@ -300,7 +309,7 @@ __global__ void __launch_bounds__(kDirThreads, 2)
                 asm volatile("cp.async.commit_group;" ::: "memory");
             };
             __syncthreads();   // the rows' offsets
-            if (j_first < j_end) stage(j_first, 0);
+            stage(j_first, 0);
             int buf = 0;
             for (long long j0 = j_first; j0 < j_end; j0 += tile, buf ^= 1) {
                 const int cnt = (int)min((long long)tile, j_end - j0);
@@ -354,9 +363,14 @@ __global__ void __launch_bounds__(kDirThreads, 2)
                 two_add(s, e, v4[f]);
                 e += v4[32 * 4 + f];
             }
+            if constexpr (TURN) {
+                two_add(tot[u], err[u], s);
+                err[u] += e;
+                continue;
+            }
             const long long k = direct_node(T, b, i);
             if (k < 0) continue;
-            if (nsplit == 1) {
+            if (T.parts == 1) {
                 direct_store(T, out, f, k, s + e, inv_c);
                 continue;
             }
@@ -365,28 +379,35 @@ __global__ void __launch_bounds__(kDirThreads, 2)
             w[T.n] = e;
         }
     }
+    if constexpr (!TURN) return;
+#pragma unroll
+    for (int u = 0; u < kDirOut; ++u) {
+        const int c = threadIdx.x + u * kDirThreads;
+        const long long k = direct_node(T, b, c % kDirTargets);
+        if (k >= 0) direct_store(T, out, c / kDirTargets, k, tot[u] + err[u], inv_c);
+    }
 }
 
 // The parts of each target in order (32 B per node and part, a few percent of
 // the sums' time).
 __global__ void __launch_bounds__(kDirThreads)
     k_direct_sum(const DirectTarget *__restrict__ tgts, int ntgt, OutPtrs out, const float *__restrict__ part,
-                 int nsplit, float inv_c)
+                 float inv_c)
 {
     int lo = 0, hi = ntgt;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (tgts[mid].block0 <= (int)blockIdx.x) lo = mid; else hi = mid;
+        if (tgts[mid].sum0 <= (int)blockIdx.x) lo = mid; else hi = mid;
     }
     const DirectTarget &T = tgts[lo];
-    const int b = (int)blockIdx.x - T.block0;
+    const int b = (int)blockIdx.x - T.sum0;
 #pragma unroll
     for (int u = 0; u < kDirOut; ++u) {
         const int c = threadIdx.x + u * kDirThreads, f = c / kDirTargets;
         const long long k = direct_node(T, b, c % kDirTargets);
         if (k < 0) continue;
         float s = 0.0f, e = 0.0f;
-        for (int i = 0; i < nsplit; ++i) {
+        for (int i = 0; i < T.parts; ++i) {
             const float *w = part + T.part0 + ((long long)i * 4 + f) * 2 * T.n + k;
             two_add(s, e, w[0]);
             e += w[T.n];
@@ -427,30 +448,39 @@ int direct_blocks(const int n[3], int groups)
     return (int)((places + kDirTargets - 1) / kDirTargets);
 }
 
-// Parts of the sources: enough blocks for sixteen per SM, so that blocks of
-// unequal length leave no long tail, each with at least 512 sources.
-int direct_splits(int blocks, long long min_sources)
+// Parts of a target's sources: enough blocks for eight per SM of a 152-SM
+// device, so that blocks of unequal length leave no long tail, each part with
+// at least 512 sources.  From the target and its own sources alone: the order
+// of its sum, so its bits, are the same whatever else a context holds, on any
+// device, and with or without room for the workspace.
+int direct_parts(int blocks, long long sources)
 {
-    const long long want = (16 * 152 + blocks - 1) / (blocks > 0 ? blocks : 1), most = min_sources / 512;
+    const long long want = (8 * 152 + blocks - 1) / (blocks > 0 ? blocks : 1), most = sources / 512;
     const long long s = want < most ? want : most;
     return (int)(s < 1 ? 1 : s > 64 ? 64 : s);
 }
 
 cudaError_t open_direct_smem_limit(int max_optin)
 {
-    return cudaFuncSetAttribute(k_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
+    cudaError_t e = cudaFuncSetAttribute(k_direct<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
+    return e ? e : cudaFuncSetAttribute(k_direct<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
 }
 
 cudaError_t launch_direct(const DirectTarget *d_tgts, int ntgt, const DirectPair *d_pairs, const OutPtrs &out,
-                          float *part, int nsplit, int nblocks, int max_nlag, long long step, int clamp,
-                          float inv_c, cudaStream_t s)
+                          float *part, bool turn, int nblocks, int sum_blocks, int max_nlag, long long step,
+                          int clamp, float inv_c, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
-    k_direct<<<dim3(nblocks, nsplit), kDirThreads, direct_smem(max_nlag, direct_tile_of(max_nlag)), s>>>(
-        d_tgts, ntgt, d_pairs, out, part, direct_tile_of(max_nlag), max_nlag, step, clamp, inv_c);
+    const int tile = direct_tile_of(max_nlag);
+    const auto go = [&](auto kern) {
+        kern<<<nblocks, kDirThreads, direct_smem(max_nlag, tile), s>>>(d_tgts, ntgt, d_pairs, out, part, tile, max_nlag,
+                                                                       step, clamp, inv_c);
+    };
+    if (turn) go(k_direct<true>);
+    else go(k_direct<false>);
     cudaError_t e = cudaGetLastError();
-    if (e || nsplit == 1) return e;
-    k_direct_sum<<<nblocks, kDirThreads, 0, s>>>(d_tgts, ntgt, out, part, nsplit, inv_c);
+    if (e || sum_blocks <= 0) return e;
+    k_direct_sum<<<sum_blocks, kDirThreads, 0, s>>>(d_tgts, ntgt, out, part, inv_c);
     return cudaGetLastError();
 }
 

@@ -113,10 +113,12 @@ struct DirectTarget {
     long long n;
     double ht;
     int p0, p1;              // DirectPair range
-    int block0;              // first block in the direct grid
+    long long sources;       // source nodes over its pairs
+    int blocks, parts;       // blocks over its nodes, parts of its sources (direct_parts)
+    int block0, sum0;        // first block in the direct grid and in that of the parts' sums
     int accumulate;          // add onto the output (FFT pairs wrote it) instead of writing
     int groups, shared;      // groups of four nodes per row (0: consecutive nodes); they share samples
-    long long part0;         // its parts' first float in the workspace ([split][4][hi, lo][n])
+    long long part0;         // its parts' first float in the workspace ([part][4][hi, lo][n])
     const long long *d_step; // the step, for launches made with step < 0 (graph replay)
 };
 
@@ -268,13 +270,13 @@ cudaError_t launch_fwd_plane_line(int M, const FwdRing *d_rings, const IoPtrs &i
                                   int nblocks, size_t smem, int far_slot, cudaStream_t s);
 cudaError_t launch_inv_plane_line(int M, const InvTarget *d_tgts, int t0, int t1, int block_lo, const OutPtrs &out,
                                   int nblocks, size_t smem, float inv_c, long long step, cudaStream_t s);
-// part: the workspace of nsplit parts of the sources per target (unused for one)
+// part: the workspace of the targets' parts; turn: there is none, every block runs its targets' parts in turn
 cudaError_t launch_direct(const DirectTarget *d_tgts, int ntgt, const DirectPair *d_pairs,
-                          const OutPtrs &out, float *part, int nsplit, int nblocks, int max_nlag, long long step,
-                          int clamp, float inv_c, cudaStream_t s);
+                          const OutPtrs &out, float *part, bool turn, int nblocks, int sum_blocks, int max_nlag,
+                          long long step, int clamp, float inv_c, cudaStream_t s);
 int direct_groups(int nx, double h, double cdt, bool *shared);
 int direct_blocks(const int n[3], int groups);
-int direct_splits(int blocks, long long min_sources);
+int direct_parts(int blocks, long long sources);
 cudaError_t open_direct_smem_limit(int max_optin);
 constexpr int kDirMaxLags = 226;   // longest lag window of a direct pair
 

@@ -1,6 +1,7 @@
-"""The direct sum's precision against the FP64 oracle: exact geometry where
-the grid's numbers are exact, a compensated sum, any unit of length and speed
-of light."""
+"""The direct sum's precision and its order, against the FP64 oracle: exact
+geometry where the grid's numbers are exact, a compensated sum, any unit of
+length and speed of light, and the same bits with and without the workspace
+of its parts."""
 import numpy as np
 import pytest
 
@@ -73,3 +74,37 @@ def test_any_unit_of_length_and_speed(unit, c):
         scale = np.linalg.norm(want[:, :1]), np.linalg.norm(want[:, 1:])   # A carries 1 / c
         assert np.linalg.norm(got.T[:, :1] - want[:, :1]) <= 1e-6 * scale[0]
         assert np.linalg.norm(got.T[:, 1:] - want[:, 1:]) <= 1e-6 * scale[1]
+
+
+CASES = {   # domains, mode: parts for both targets, for one only (a small one under a large source), for none
+    "parts": ([synth.Domain((0.0, 0.0, 0.0), (20, 19, 18), 0.25), synth.Domain((6.0, 0.4, -0.3), (17, 13, 11), 0.3)],
+              rp.RP_MODE_DIRECT),
+    "one_target": ([synth.Domain((0.0, 0.0, 0.0), (24, 23, 22), 0.25), synth.Domain((7.0, 0.4, -0.3), (5, 4, 3), 0.3)],
+                   rp.RP_MODE_FFT),
+    "no_parts": ([synth.Domain((0.0, 0.0, 0.0), (9, 8, 5), 0.25), synth.Domain((3.5, 0.4, -0.3), (5, 4, 3), 0.3)],
+                 rp.RP_MODE_DIRECT),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_same_bits_without_the_workspace(name):
+    """Under a device budget there is no workspace and a block runs its
+    targets' parts in turn: the same bits; both against the oracle."""
+    import torch
+    dev = torch.device("cuda", 0)
+    doms, mode = CASES[name]
+    hists = _noise(doms, 7)
+    got = []
+    for budget in (0, 1 << 33):
+        with rp.RetardedPotentials(doms, synth.C_AU, 0.05, mode=mode, device_budget=budget) as lib:
+            for i in range(7):
+                x = [torch.from_numpy(h[i]).to(dev) for h in hists]
+                lib.push_all([v[0].contiguous() for v in x], [v[1:].contiguous().reshape(-1) for v in x])
+            phi, A = lib.evaluate()
+            got.append([np.concatenate([phi[t].cpu().numpy()[None], A[t].cpu().numpy().reshape(3, -1)])
+                        for t in range(len(doms))])
+    for t, d in enumerate(doms):
+        np.testing.assert_array_equal(got[0][t], got[1][t])
+        nodes = np.arange(0, d.N, max(1, d.N // 400))
+        want = oracle_values(doms, hists, 0, synth.C_AU, 0.05, t, 6, nodes)
+        assert _joint(got[0][t][:, nodes], want) <= 2e-6    # FP32 tau at a spacing that is not exact
