@@ -176,10 +176,16 @@ def _ptr(x) -> int:
 
 
 def _ptr_array(xs: Sequence):
-    """The argument for a pointer-array parameter (ctypes passes an array as
-    the address of its first element) and what must outlive the call."""
-    arr = xs if isinstance(xs, ctypes.Array) else pointer_array(xs)   # made by pointer_array, or now
-    return arr, arr
+    """The argument for a pointer-array parameter (ctypes passes an array of
+    c_void_p as the address of its first element; arrays of other pointers or
+    of addresses as integers are cast) and what must outlive the call."""
+    if not isinstance(xs, ctypes.Array):
+        xs = pointer_array(xs)
+    if xs._type_ is ctypes.c_void_p:
+        return xs, xs
+    if ctypes.sizeof(xs._type_) != ctypes.sizeof(ctypes.c_void_p):
+        raise ValueError("a pointer array must hold addresses")
+    return ctypes.cast(xs, _PP), xs
 
 
 def pointer_array(xs: Sequence):
