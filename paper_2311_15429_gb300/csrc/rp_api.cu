@@ -1534,7 +1534,7 @@ rp_status enqueue_push(rp_ctx *ctx, int d0, int d1, const IoPtrs &in)
     }
     for (const LaunchGroup &g : launches) {
         if ((st = timed_launch(ctx, RP_K_FWD_COLUMN, "forward column pass", [&] {
-                 return launch_fwd_column(column_class(g.cls), rings, g.i0, g.i1, g.blk2_0, g.blk2_1 - g.blk2_0,
+                 return launch_fwd_column(g.cls, rings, g.i0, g.i1, g.blk2_0, g.blk2_1 - g.blk2_0,
                                           ctx->smem_col, kstep, ctx->stream);
              })))
             return st;

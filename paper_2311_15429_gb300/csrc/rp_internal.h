@@ -252,7 +252,7 @@ cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, i
                              cudaStream_t s);
 cudaError_t launch_fwd_plane(int plane_class, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
                              int block_lo, int nblocks, size_t smem, int far_slot, cudaStream_t s);
-cudaError_t launch_fwd_column(int column_class, const FwdRing *d_rings, int r0, int r1, int block_lo,
+cudaError_t launch_fwd_column(int size_class, const FwdRing *d_rings, int r0, int r1, int block_lo,
                               int nblocks, size_t smem, long long step, cudaStream_t s);
 cudaError_t launch_mac_inv_column(bool comp, const InvTarget *d_tgts, int t0, int t1, int block_lo,
                                   const MacEntry *d_entries, int nblocks, size_t smem, long long step,

@@ -160,7 +160,7 @@ static rp_status spill_transform(rp_ctx *ctx, int w0, int w1, long long j)
          })))
         return st;
     return timed_launch(ctx, RP_K_FWD_COLUMN, "window forward column pass", [&] {
-        return launch_fwd_column(column_class(cls), ctx->d_wfwd, w0, w1, F0.tile0, tiles, ctx->smem_col, j, ctx->stream);
+        return launch_fwd_column(cls, ctx->d_wfwd, w0, w1, F0.tile0, tiles, ctx->smem_col, j, ctx->stream);
     });
 }
 
