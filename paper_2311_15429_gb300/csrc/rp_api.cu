@@ -146,7 +146,9 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
     for (LaunchGroup &g : ctx->inv_groups) {
         const int cls = column_class(g.cls);
         if (cls == 0) continue;
-        g.fields = mac_tma_fields(cls, ctx->comp, g.blk1 - g.blk0, ctx->sm_count);
+        const int ntiles = g.blk1 - g.blk0;
+        const double entries = (double)(ctx->inv[g.i1 - 1].e1 - ctx->inv[g.i0].e0) / (g.i1 - g.i0);
+        g.fields = mac_tma_fields(cls, ctx->comp, ntiles, entries, ctx->sm_count);
         // two targets that read the same ring at the same lag; same tiles in all
         std::map<std::pair<const float2 *, int>, int> reader;
         bool shared = false, same = true;
@@ -159,8 +161,7 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
             }
         }
         g.share = shared && same;
-        g.fft_warps = mac_tma_fft_warps(cls, ctx->comp, g.fields,
-                                        (double)(ctx->inv[g.i1 - 1].e1 - ctx->inv[g.i0].e0) / (g.i1 - g.i0));
+        g.fft_warps = mac_tma_fft_warps(cls, ctx->comp, g.fields, ntiles, entries, ctx->sm_count);
         g.stages = mac_tma_stages(cls, max_optin, g.fields);
         if (ctx->cfg.mac_stages >= 2) g.stages = std::min(g.stages, ctx->cfg.mac_stages);
         if (g.stages < 2) {

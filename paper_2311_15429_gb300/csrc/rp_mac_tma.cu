@@ -201,22 +201,26 @@ __device__ __forceinline__ void column_tile_store(float2 *acc, const float2 *tw,
 // Warps of the inverse column FFT (FW): seven beside the plain sum's MAC
 // warps; beside the compensated ones, whose accumulators need the registers,
 // three, which keep up with tiles of many entries and leave the multiply-adds
-// the issue slots.  Tiles of few entries (the self lags alone) wait for them:
-// there as many as the registers leave, seven up to M = 64 and five at 96 (at
-// 128 and 192 none are left).  32 x 48^3, 4 entries a tile: MAC 382 us with
-// three, 354 with five; 2 x 48^3, 9 entries: 52.6 and 54.4; 64^3 class of the
-// mixed sizes, 4 entries: 27.3 with three, 25.9 with seven; four 27^3
-// neighbours, 19 entries: 62.2 and 66.1.
+// the issue slots.  Tiles of few entries (the self lags alone) wait for them
+// where a block has several: there as many as the registers leave, seven at
+// M = 64 and five at 96 (at 128 and 192 none are left; 32 and 48 transform as
+// fast with three).  32 x 48^3, 4 entries a tile: MAC 382 us with three, 354
+// with five; 2 x 48^3, 9 entries: 52.6 and 54.4; 64^3 class of the mixed
+// sizes, 4 entries: 27.3 with three, 25.9 with seven; four 27^3 neighbours, 19
+// entries: 62.2 and 66.1; four far 24^3, 3 entries: the step 39.1 with three,
+// 41.0 with seven.  A block's last unit is every warp's: with one unit a block
+// (one 24^3) 17.9 with three, 23.1 with seven.
 constexpr int kFewEntries = 6;
-__host__ __device__ constexpr int few_fft_warps(int M) { return M <= 64 ? 7 : M == 96 ? 5 : 3; }
+__host__ __device__ constexpr int few_fft_warps(int M) { return M == 64 ? 7 : M == 96 ? 5 : 3; }
 
 // A block's unit of work is FH fields of one tile: all four (the kernel tile
 // read once), unless
 //   * M = 192, compensated: a MAC thread would hold 128 floats of sums and
 //     compensation for four fields and spill them, so a unit is two;
-//   * the plan's tiles are so few that half of the SMs would have none
-//     (elongated and small grids): two fields or one, the kernel tile then
-//     read again from L2 by the neighbouring block (mac_tma_fields).
+//   * the plan's tiles are so few that half of the SMs would have none, and
+//     not of the smallest (elongated and small grids): two fields or one, the
+//     kernel tile then read again from L2 by the neighbouring block
+//     (mac_tma_fields).
 // Every field is summed in the same order whatever the unit.
 //
 // Units go target by target, except (share) where the targets of a launch
@@ -573,19 +577,23 @@ cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_
 // 128, 40 entries): 54.7 us per step with four fields, 44.2 with two; one 8 x
 // 8 x 90 box (17 tiles of M = 192): 40.3 with two, 33.5 with one.  Beyond one
 // unit per SM the shorter copies only cost (16 x 16 x 96 pair: 67.7 with two,
-// 80.6 with one).
-int mac_tma_fields(int M, bool comp, int ntiles, int sms)
+// 80.6 with one), and so they do where a tile's entries are read in about 3 us
+// by one block: two 14^3 (6 entries of 20 KB) 20.5 with two fields, 18.3 with
+// four; one 20^3 (3 of 30 KB) 18.2 and 17.0; two 16^3 (7 of 20 KB) 17.9 and
+// 22.2; one 16 x 16 x 33 box (4 of 60 KB) 16.2 with one, 20.3 with four.
+int mac_tma_fields(int M, bool comp, int ntiles, double entries, int sms)
 {
     int fh = unit_runs(M, 4, comp) ? 4 : 2;
+    if (entries * 5 * M * 128 <= 128 * 1024) return fh;   // kernel and four field tiles of M x 16 an entry
     while (fh > 1 && ntiles * (4 / fh) * 2 <= sms) fh /= 2;
     return fh;
 }
 
 // FFT warps of a launch whose targets have `entries` (source, lag) terms on average.
-int mac_tma_fft_warps(int M, bool comp, int fh, double entries)
+int mac_tma_fft_warps(int M, bool comp, int fh, int ntiles, double entries, int sms)
 {
     if (!comp) return kFftWarps;
-    return fh == 4 && entries <= kFewEntries ? few_fft_warps(M) : 3;
+    return fh == 4 && ntiles > sms && entries <= kFewEntries ? few_fft_warps(M) : 3;
 }
 
 int mac_tma_stages(int M, int smem_optin, int fh)
