@@ -820,19 +820,29 @@ cudaError_t launch_fwd_plane(int cls, const FwdRing *d_rings, const IoPtrs &in, 
     }
 }
 
+// The general column and MAC kernels hold 552 B of shared memory per point
+// along z and run for tens of microseconds in few blocks: launched while the
+// kernel before still holds the SMs, several land on an SM that has room,
+// beside idle ones, and which step that hits changes with every other kernel's
+// size.  From 64 points along z (of the longest target: the plan's shared
+// memory) they start after it.  9 x 9 x 33 box: step 67 -> 47 us (12 x 12 x 64
+// 65 -> 63, two 6 x 6 x 48 69 -> 57, two 9 x 9 x 96 135 -> 126); at 48 points
+// and fewer the launch gap costs more than it gives (6 x 6 x 20 22.5 -> 26.7).
+constexpr size_t kGeneralApart = 64 * sizeof(float2) * (1 + 4 * kTileYPad);
+
 cudaError_t launch_fwd_column(int cls, const FwdRing *d_rings, int r0, int r1, int block_lo, int nblocks,
                               size_t smem, long long step, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
     const int M = column_class(cls);
-    const bool cube = M > 0 && plane_class(cls) == M;
+    const bool cube = M > 0 && plane_class(cls) == M, overlap = M > 0 || smem < kGeneralApart;
     if (tile16_class(M)) smem = smem_fwd_column16(M);
     const dim3 threads(tile16_class(M) ? kColumn16Threads : kColumnThreads);
     switch (M) {
 #define X(M)                                                                                                  \
     case M:                                                                                                   \
-        return launch_pdl(cube ? fwd_column_kernel<M, (M > 0)>() : fwd_column_kernel<M, false>(), dim3(nblocks), \
-                          threads, smem, s, d_rings, r0, r1, block_lo, step);
+        return launch_kernel(overlap, cube ? fwd_column_kernel<M, (M > 0)>() : fwd_column_kernel<M, false>(), \
+                             dim3(nblocks), threads, smem, s, d_rings, r0, r1, block_lo, step);
         RP_COLUMN_CLASSES(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -844,8 +854,8 @@ cudaError_t launch_mac_inv_column(bool comp, const InvTarget *d_tgts, int t0, in
                                   cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
-    return launch_pdl(comp ? k_mac_inv_column<true> : k_mac_inv_column<false>, dim3(nblocks), dim3(kThreads), smem, s,
-                      d_tgts, t0, t1, block_lo, d_entries, step, clamp);
+    return launch_kernel(smem < kGeneralApart, comp ? k_mac_inv_column<true> : k_mac_inv_column<false>, dim3(nblocks),
+                         dim3(kThreads), smem, s, d_tgts, t0, t1, block_lo, d_entries, step, clamp);
 }
 
 cudaError_t launch_inv_plane(int cls, const InvTarget *d_tgts, int t0, int t1, int block_lo, const OutPtrs &out,
