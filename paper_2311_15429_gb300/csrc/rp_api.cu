@@ -1058,6 +1058,10 @@ rp_status rp_finalize(rp_ctx *ctx)
     });
     std::vector<int> ring_pos(ring_keys.size());
     std::map<int, const float2 *> tw;
+    int blocks32 = 0;
+    for (size_t r = 0; r < ring_keys.size(); ++r)
+        if (plane_class(ring_class((int)r)) == 32) blocks32 += 4 * ctx->doms[ring_keys[r].first].n[2];
+    ctx->lane32 = blocks32 <= kLanePlane32;
     for (size_t i = 0; i < ring_order.size(); ++i) {
         const int r = ring_order[i];
         ring_pos[r] = (int)i;
@@ -1528,7 +1532,8 @@ rp_status enqueue_push(rp_ctx *ctx, int d0, int d1, const IoPtrs &in)
     for (const LaunchGroup &g : launches) {
         const int cls = plane_class(g.cls);
         if ((st = timed_launch(ctx, RP_K_FWD_PLANE, "forward plane pass", [&] {
-                 return launch_fwd_plane(cls, rings, fin, g.i0, g.i1, g.blk0, g.blk1 - g.blk0, ctx->smem_plane_cls[class_slot(cls)],
+                 return launch_fwd_plane(cls, ctx->lane32, rings, fin, g.i0, g.i1, g.blk0, g.blk1 - g.blk0,
+                                         ctx->smem_plane_cls[class_slot(cls)],
                                          (int)(step % std::max(1, ctx->cfg.far_batch)), ctx->stream);
              })))
             return st;

@@ -171,6 +171,7 @@ struct rp_ctx {
     int dir_nlag = 0, dir_sum_blocks = 0;            // direct sums: longest lag window, blocks that add the parts
     float *dir_part = nullptr;                       // their workspace (a target with more than one part)
     bool dir_turn = false;                           // no workspace though a target has: parts in turn
+    bool lane32 = false;                             // forward plane passes at 32 points: the form for few blocks
     size_t smem_plane_cls[7] = {}, smem_inv_cls[7] = {}; // plane passes' shared memory per launch (by class_slot)
     int max_lag = 0, raw_depth = 0, spec_depth = 0;
     long long spectral_bytes = 0, kernel_bytes = 0, device_bytes = 0;

@@ -17,10 +17,13 @@
 // The column pass runs the two-stage shared-memory tile transform of
 // rp_fft.cuh for 64, 96, 128 and 192 points along z (k_fwd_column16) and the
 // lane-shuffle line transform otherwise; the plane passes here (lane-shuffle
-// lines) serve a cross-section of 48 and, with M = 0, any supported shape read
-// at run time; the other square ones are in rp_plane.cu.  The MAC here serves
+// lines) serve a cross-section of 48, with M = 0 any supported shape read at
+// run time, and the smallest forward launches at 32; the other square ones are
+// in rp_plane.cu.  The MAC here serves
 // shapes with no column class.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "rp_fft.cuh"
 #include "rp_internal.h"
@@ -738,11 +741,12 @@ int size_class(const Axis &ax, const Axis &ay, const Axis &az)
 
 size_t smem_fwd_plane(int cls, int ny, const Axis &ax)
 {
-    if (plane_line_class(cls)) return smem_fwd_plane_line(cls, ny);
+    const size_t line = plane_line_class(cls) ? smem_fwd_plane_line(cls, ny) : 0;
+    if (line && cls != 32) return line;   // 32: either form
     const int kx = ax.M / 2 + 1;
     const int qs = kx | 1;
     // twiddles (x and y, bounded by kMaxFFT each) + Q + per-group scratch
-    return sizeof(float2) * (2 * kMaxFFT + (size_t)ny * qs + (size_t)(kPlaneThreads / 32) * 32 * ax.R);
+    return std::max(line, sizeof(float2) * (2 * kMaxFFT + (size_t)ny * qs + (size_t)(kPlaneThreads / 32) * 32 * ax.R));
 }
 
 size_t smem_fwd_column(const Axis &az) { return sizeof(float2) * ((size_t)az.M + 4 * (size_t)az.M * kTileYPad); }
@@ -784,6 +788,7 @@ cudaError_t open_kernel_smem_limits(int max_optin)
     if ((e = open(k_fwd_plane<M>)) || (e = open(k_inv_plane<M>))) return e;
     RP_PLANE_CLASSES(X)
 #undef X
+    if ((e = open(k_fwd_plane<32>))) return e;
 #define X(M) \
     if ((e = open(fwd_column_kernel<M, false>())) || (e = open(fwd_column_kernel<M, (M > 0)>()))) return e;
     RP_COLUMN_CLASSES(X)
@@ -803,13 +808,16 @@ cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_plane(int cls, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1, int block_lo,
+cudaError_t launch_fwd_plane(int cls, bool lane32, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1, int block_lo,
                              int nblocks, size_t smem, int far_slot, cudaStream_t s)
 {
     if (nblocks <= 0) return cudaSuccess;
-    if (plane_line_class(cls))
+    if (plane_line_class(cls) && !(lane32 && cls == 32))
         return launch_fwd_plane_line(cls, d_rings, in, r0, r1, block_lo, nblocks, smem, far_slot, s);
     switch (cls) {
+    case 32:
+        return launch_pdl(k_fwd_plane<32>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_rings, in, r0, r1, block_lo,
+                          far_slot);
 #define X(M)                                                                                                      \
     case M:                                                                                                       \
         return launch_pdl(k_fwd_plane<M>, dim3(nblocks), dim3(kPlaneThreads), smem, s, d_rings, in, r0, r1,       \

@@ -250,7 +250,13 @@ inline int column_class(int size_class) { return size_class >> 8; }
 cudaError_t launch_ring_push(const RawRing *d_rings, const IoPtrs &in, int d0, int d1,
                              const int *h_block0, int nblocks, long long step,
                              cudaStream_t s);
-cudaError_t launch_fwd_plane(int plane_class, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
+// A plan with at most kLanePlane32 forward plane blocks at 32 points (lane32)
+// runs the lane-shuffle lines there: all latency, and theirs is the shorter
+// (one 16^3, 64 blocks: step 16.0 -> 13.9 us, one 16 x 16 x 8 18.0 -> 16.1); at
+// 128 blocks (two 16^3) rp_plane.cu's lines take 18.0, these 21.3.  From the
+// plan, not the launch, so that every way to push gives the same bits.
+constexpr int kLanePlane32 = 64;
+cudaError_t launch_fwd_plane(int plane_class, bool lane32, const FwdRing *d_rings, const IoPtrs &in, int r0, int r1,
                              int block_lo, int nblocks, size_t smem, int far_slot, cudaStream_t s);
 cudaError_t launch_fwd_column(int size_class, const FwdRing *d_rings, int r0, int r1, int block_lo,
                               int nblocks, size_t smem, long long step, cudaStream_t s);
