@@ -231,7 +231,7 @@ typedef struct {
     int mac_tma;              /* 1: the spectral MAC of targets with a compiled length along z is fed by TMA copies */
     int npairs_far;           /* pairs on the low-rank far path */
     long long far_bytes;      /* device memory of the far path (factors, batches, rings) */
-    int mac_warps;            /* consumer warps of the MAC variant in use (last size class), 0 if none */
+    int mac_warps;            /* consumer warps of the MAC variant in use (its last launch of a step), 0 if none */
     int npairs_learned;       /* pairs on the learned far path (after rp_train_far_model) */
     int spill_windows;        /* RP_FLAG_HISTORY_SPILL: lag windows read from host-refilled window rings */
     int reserved;

@@ -148,6 +148,7 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
         if (cls == 0) continue;
         const int ntiles = g.blk1 - g.blk0;
         const double entries = (double)(ctx->inv[g.i1 - 1].e1 - ctx->inv[g.i0].e0) / (g.i1 - g.i0);
+        g.mac_warps = ctx->comp ? kCompWarps : ctx->cfg.mac_warps ? ctx->cfg.mac_warps : 16;
         g.fields = mac_tma_fields(cls, ctx->comp, ntiles, entries, ctx->sm_count);
         // two targets that read the same ring at the same lag; same tiles in all
         std::map<std::pair<const float2 *, int>, int> reader;
@@ -769,24 +770,20 @@ rp_status plan_direct(rp_ctx *ctx)
 
 // Launch-shape autotuning: time each consumer-warp variant of the TMA-fed MAC
 // on this plan (two launches after one warm-up, on the context stream, over
-// rings whose contents do not matter for timing) and keep the fastest per
-// size class.  Every variant reads the same data and sums in the same order.
+// rings whose contents do not matter for timing) and keep the fastest of each
+// launch (launches of one column class differ in tiles, units and stages).  Every variant reads the same data and sums in the same order.
 rp_status autotune_mac(rp_ctx *ctx)
 {
-    if (ctx->comp) {   // one compensated variant
-        std::fill(std::begin(ctx->mac_cw), std::end(ctx->mac_cw), kCompWarps);
-        return RP_OK;
-    }
-    if (!ctx->tma || ctx->cfg.mac_warps) return RP_OK;
+    if (ctx->comp || !ctx->tma || ctx->cfg.mac_warps) return RP_OK;   // compensated: one variant
     cudaEvent_t a = nullptr, b = nullptr;
     RP_CUDA(ctx, cudaEventCreate(&a));
     RP_CUDA(ctx, cudaEventCreate(&b));
     rp_status st = RP_OK;
     const long long step = ctx->max_lag;   // every (step - lag) is a valid slot
-    for (const LaunchGroup &g : ctx->inv_groups) {
+    for (LaunchGroup &g : ctx->inv_groups) {
         const int cls = column_class(g.cls);
         if (cls == 0 || st) continue;
-        const int slot = class_slot(cls), ntiles = g.blk1 - g.blk0;
+        const int ntiles = g.blk1 - g.blk0;
         float best = 1e30f;
         for (int cw : {8, 12, 16}) {
             auto go = [&] {
@@ -806,7 +803,7 @@ rp_status autotune_mac(rp_ctx *ctx)
             }
             if (ms < best) {
                 best = ms;
-                ctx->mac_cw[slot] = cw;
+                g.mac_warps = cw;
             }
         }
     }
@@ -873,7 +870,6 @@ rp_status rp_create(const rp_config *cfg, int device, void *stream, rp_ctx **out
     ctx->cfg = *cfg;
     if (ctx->cfg.far_points == 0) ctx->cfg.far_points = 4;
     if (ctx->cfg.far_batch == 0) ctx->cfg.far_batch = 32;
-    if (ctx->cfg.mac_warps) std::fill(std::begin(ctx->mac_cw), std::end(ctx->mac_cw), ctx->cfg.mac_warps);
     ctx->plan_only = (cfg->flags & RP_FLAG_PLAN_ONLY) != 0;
     ctx->split = (cfg->flags & RP_FLAG_GROUND_STATE_SPLIT) != 0;
     ctx->spill = (cfg->flags & RP_FLAG_HISTORY_SPILL) != 0;
@@ -1941,7 +1937,7 @@ static rp_status evaluate_launches(rp_ctx *ctx, const OutPtrs &out, long long st
         const int ntiles = g.blk1 - g.blk0;
         if ((st = timed_launch(ctx, RP_K_MAC_INV_COLUMN, "MAC + inverse column pass", [&] {
                  if (const int cls = column_class(g.cls); ctx->tma && cls > 0)
-                     return launch_mac_tma(cls, ctx->mac_cw[class_slot(cls)], ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0,
+                     return launch_mac_tma(cls, g.mac_warps, ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0,
                                            ntiles, g.share, ctx->d_entries, kstep, clamp, g.fields, g.fft_warps,
                                            g.stages, ctx->sm_count, ctx->d_err, ctx->stream);
                  return launch_mac_inv_column(ctx->comp, ctx->d_inv, g.i0, g.i1, g.blk0, ctx->d_entries, ntiles,
@@ -2533,7 +2529,7 @@ rp_status rp_query(rp_ctx *ctx, rp_stats *out)
     for (const PairPlan &p : ctx->pairs) out->npairs_other += p.kind == RP_PAIR_OTHER;
     out->mac_warps = 0;
     for (const LaunchGroup &g : ctx->inv_groups)
-        if (column_class(g.cls) > 0 && ctx->tma) out->mac_warps = ctx->mac_cw[class_slot(column_class(g.cls))];
+        if (column_class(g.cls) > 0 && ctx->tma) out->mac_warps = g.mac_warps;
     out->npairs_direct = 0;
     out->npairs_fft = 0;
     for (const PairPlan &p : ctx->pairs) {

@@ -58,7 +58,7 @@ struct LaunchGroup {
     int blk0, blk1;
     int blk2_0, blk2_1;
     int fields = 0, stages = 0;   // MAC launches: fields of a block's unit, field stages of its pipeline,
-    int fft_warps = 0;            // warps of its inverse FFT
+    int mac_warps = 0, fft_warps = 0;   // its multiply-add and inverse-FFT warps
     bool share = false;           // MAC launches: targets with the same tiles that read the same source slots
 };
 
@@ -183,8 +183,7 @@ struct rp_ctx {
     DirectTarget *d_dtg = nullptr;
     DirectPair *d_dpairs = nullptr;
     RawRing *d_raw = nullptr;
-    bool tma = false;                // TMA-fed MAC available for the cubic classes
-    int mac_cw[7] = {16, 16, 16, 16, 16, 16, 16};   // consumer warps of the MAC per class
+    bool tma = false;                // TMA-fed MAC in use where a target has a column class
     int sm_count = 0;
     int *d_err = nullptr;            // set by a kernel whose bounded wait ran out
     // far pairs (low-rank path)

@@ -36,3 +36,25 @@ def test_small_plans(name, plain):
         want = oracle_values(doms, hists, 0, synth.C_AU, 0.05, t, T - 1, nodes)
         errs = rel_l2(res[T - 1][t][:, nodes], want)
         assert max(errs) <= TOL, (name, t, errs)
+
+
+@pytest.mark.parametrize("warps", [0, 8])
+@pytest.mark.parametrize("plain", [False, True])
+def test_launches_of_one_column_class(plain, warps):
+    """A cube and a box of the same padded length along z are two MAC launches,
+    each with warps of its own."""
+    if warps and not plain:
+        pytest.skip("the compensated sum has one variant")
+    doms = [synth.Domain((0.0, 0.0, 0.0), (25, 26, 27), 0.3), synth.Domain((9.0, 0.4, -0.2), (14, 15, 28), 0.3)]
+    flags = rp.RP_FLAG_PLAIN_SUM if plain else 0
+    with rp.RetardedPotentials(doms, synth.C_AU, 0.05, flags=flags, mac_warps=warps) as lib:
+        T = lib.query()["max_lag"] + 3
+        used = lib.query()["mac_warps"]
+    assert used == (warps or used) and used in ((8, 12, 16) if plain else (12,))
+    hists = histories(synth.seeded_sources(doms), 0, T, 0.05)
+    res = run_library(doms, synth.C_AU, 0.05, hists, 0, [T - 1], flags=flags, mac_warps=warps)
+    for t, d in enumerate(doms):
+        nodes = np.arange(0, d.N, max(1, d.N // 1500))
+        want = oracle_values(doms, hists, 0, synth.C_AU, 0.05, t, T - 1, nodes)
+        errs = rel_l2(res[T - 1][t][:, nodes], want)
+        assert max(errs) <= TOL, (t, errs)
