@@ -1215,7 +1215,10 @@ rp_status rp_finalize(rp_ctx *ctx)
             ctx->dtg.push_back(D);
         }
     }
-    if (max_nlag > 600) return fail(ctx, RP_ERR_UNSUPPORTED, "direct pair lag window above 600 steps");
+    // the kernel's limit; a plan alone takes longer windows
+    if (const int most = ctx->plan_only ? kDirPlanLags : kDirMaxLags; max_nlag > most)
+        return fail(ctx, RP_ERR_UNSUPPORTED, "direct pair lag window of " + std::to_string(max_nlag) +
+                                                 " steps, above " + std::to_string(most));
     // FP64 audit: every source keeps its raw slices as deep as its deepest pair reads
     if (ctx->cfg.flags & RP_FLAG_AUDIT)
         for (int t = 0; t < nd; ++t)
@@ -1272,8 +1275,6 @@ rp_status rp_finalize(rp_ctx *ctx)
     ctx->smem_optin = max_optin;
     {
         const size_t need = std::max({ctx->smem_plane, ctx->smem_col, ctx->smem_mac, ctx->smem_inv});
-        if (max_nlag > kDirMaxLags)
-            return fail(ctx, RP_ERR_UNSUPPORTED, "direct pair lag window above " + std::to_string(kDirMaxLags) + " steps");
         if (need > (size_t)max_optin)
             return fail(ctx, RP_ERR_UNSUPPORTED, "kernel shared memory " + std::to_string(need) +
                                                      " B exceeds the device limit " + std::to_string(max_optin));

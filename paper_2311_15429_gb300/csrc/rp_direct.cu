@@ -416,19 +416,20 @@ __global__ void __launch_bounds__(kDirThreads)
     }
 }
 
-size_t direct_smem(int nlag, int tile)
+constexpr size_t direct_smem(int nlag, int tile)
 {
     return 16 * (size_t)direct_elems(nlag, tile) + 8 * (size_t)(nlag + 3);
 }
 
-// The largest tile of which three blocks fit an SM (larger tiles stage more
-// per barrier); for the longest lag windows, one that fits at all.
-int direct_tile_of(int nlag)
+// The largest tile of which three blocks would fit an SM (larger tiles stage
+// more per barrier); for the longest lag windows, one that fits at all.
+constexpr int direct_tile_of(int nlag)
 {
     for (int tile : {128, 64})
         if (direct_smem(nlag, tile) <= 72 * 1024) return tile;
     return direct_smem(nlag, 32) <= 200 * 1024 ? 32 : 16;
 }
+static_assert(direct_smem(kDirMaxLags, direct_tile_of(kDirMaxLags)) <= 227 * 1024, "the longest window fits a block");
 
 }  // namespace
 

@@ -284,7 +284,9 @@ int direct_groups(int nx, double h, double cdt, bool *shared);
 int direct_blocks(const int n[3], int groups);
 int direct_parts(int blocks, long long sources);
 cudaError_t open_direct_smem_limit(int max_optin);
-constexpr int kDirMaxLags = 226;   // longest lag window of a direct pair
+// Longest lag window of a direct pair: in a context that runs (its smallest
+// tile's samples then take 124 KB of shared memory), and in a plan alone.
+constexpr int kDirMaxLags = 226, kDirPlanLags = 600;
 
 // Ground-state split and graph-replay step counter (rp_ground.cu).
 cudaError_t launch_step_advance(long long *d_step, cudaStream_t s);
