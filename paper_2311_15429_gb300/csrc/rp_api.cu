@@ -149,7 +149,7 @@ rp_status plan_mac_tma(rp_ctx *ctx, int max_optin)
         const int ntiles = g.blk1 - g.blk0;
         const double entries = (double)(ctx->inv[g.i1 - 1].e1 - ctx->inv[g.i0].e0) / (g.i1 - g.i0);
         g.mac_warps = ctx->comp ? kCompWarps : ctx->cfg.mac_warps ? ctx->cfg.mac_warps : 16;
-        g.fields = mac_tma_fields(cls, ctx->comp, ntiles, entries, ctx->sm_count);
+        g.fields = mac_tma_fields(cls, ctx->comp, ntiles, entries, g.blk2_1 - g.blk2_0, ctx->sm_count);
         // two targets that read the same ring at the same lag; same tiles in all
         std::map<std::pair<const float2 *, int>, int> reader;
         bool shared = false, same = true;

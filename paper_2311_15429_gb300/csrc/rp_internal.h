@@ -308,7 +308,7 @@ cudaError_t launch_fields(int nx, int ny, int nz, double h, double c, double dt,
 // TMA-fed MAC (rp_mac_tma.cu): column classes 32..192.  share: the launch's
 // targets have the same tiles and read some of the same source slots.
 // entries: (source, lag) terms of a target, on average
-int mac_tma_fields(int M, bool comp, int ntiles, double entries, int sms);   // fields of a block's unit of work
+int mac_tma_fields(int M, bool comp, int ntiles, double entries, int plane_blocks, int sms);   // of a block's unit
 int mac_tma_fft_warps(int M, bool comp, int fields, int ntiles, double entries, int sms);
 int mac_tma_stages(int M, int smem_optin, int fields);
 cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_t s);

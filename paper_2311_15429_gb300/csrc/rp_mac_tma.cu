@@ -217,10 +217,9 @@ __host__ __device__ constexpr int few_fft_warps(int M) { return M == 64 ? 7 : M 
 // read once), unless
 //   * M = 192, compensated: a MAC thread would hold 128 floats of sums and
 //     compensation for four fields and spill them, so a unit is two;
-//   * the plan's tiles are so few that half of the SMs would have none, and
-//     not of the smallest (elongated and small grids): two fields or one, the
-//     kernel tile then read again from L2 by the neighbouring block
-//     (mac_tma_fields).
+//   * the plan's tiles are so few that half of the SMs would have none
+//     (elongated and small grids): two fields or one, the kernel tile then
+//     read again from L2 by the neighbouring block (mac_tma_fields).
 // Every field is summed in the same order whatever the unit.
 //
 // Units go target by target, except (share) where the targets of a launch
@@ -577,14 +576,17 @@ cudaError_t launch_wait_selftest(long long limit_cycles, int *d_err, cudaStream_
 // 128, 40 entries): 54.7 us per step with four fields, 44.2 with two; one 8 x
 // 8 x 90 box (17 tiles of M = 192): 40.3 with two, 33.5 with one.  Beyond one
 // unit per SM the shorter copies only cost (16 x 16 x 96 pair: 67.7 with two,
-// 80.6 with one), and so they do where a tile's entries are read in about 3 us
-// by one block: two 14^3 (6 entries of 20 KB) 20.5 with two fields, 18.3 with
-// four; one 20^3 (3 of 30 KB) 18.2 and 17.0; two 16^3 (7 of 20 KB) 17.9 and
-// 22.2; one 16 x 16 x 33 box (4 of 60 KB) 16.2 with one, 20.3 with four.
-int mac_tma_fields(int M, bool comp, int ntiles, double entries, int sms)
+// 80.6 with one).  Nor are tiles of few entries split (160 KB, some 4 us for
+// one block) in a plan whose plane passes have fewer blocks than three quarters
+// of the SMs: those start beside the MAC, on the SMs that it leaves free, and
+// wait there.  Two 14^3 (112 plane blocks, 6 entries of 20 KB): 20.5 with two
+// fields, 18.2 with four; one 20^3 (80, 3 of 30 KB) 18.1 and 17.0; two 16^3
+// (128, 6 of 20 KB), whose blocks pile up on those SMs, 17.3 and 21.4.
+int mac_tma_fields(int M, bool comp, int ntiles, double entries, int plane_blocks, int sms)
 {
     int fh = unit_runs(M, 4, comp) ? 4 : 2;
-    if (entries * 5 * M * 128 <= 128 * 1024) return fh;   // kernel and four field tiles of M x 16 an entry
+    const double bytes = entries * 5 * M * 128;   // kernel and four field tiles of M x 16 an entry
+    if (bytes <= 160 * 1024 && 4 * plane_blocks < 3 * sms) return fh;
     while (fh > 1 && ntiles * (4 / fh) * 2 <= sms) fh /= 2;
     return fh;
 }
