@@ -86,8 +86,8 @@ DEEP = ("cfg3", "cfg4", "cfg4x8", "cfg5", "cfg5x8", "farprobe")
 # multiplies), floor and the hat weight (one subtraction), the 1/R volume
 # factor (one multiply); per field the hat interpolation (one subtraction, one
 # FMA: 3 flops), the scaling (one multiply) and the accumulation (one add),
-# 5 flops x 4 fields.  Kahan compensation (3 more adds per field) is not
-# counted: it is accuracy, not the sum.
+# 5 flops x 4 fields.  The compensation of every term (a subtraction, an FMA
+# and an addition more per field) is not counted: it is accuracy, not the sum.
 DIRECT_FLOPS_PER_PAIR_POINT = 3 + 5 + 1 + 2 + 2 + 1 + 4 * 5     # = 34
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12              # 80.6
 
@@ -646,11 +646,11 @@ def run_ours(args, rank, world, local):
             torch.cuda.synchronize()
             pms = a.elapsed_time(b) / nplain
             # ALU roofline of the direct sum: pair-points per step (every
-            # target node against every source node), 32 algorithmic flops
+            # target node against every source node), 34 algorithmic flops
             # each, against the FP32 pipes' peak at the SM clock
             pp = sum(t.N for t in w.domains) * sum(s_.N for s_ in w.domains)
             achieved = pp * DIRECT_FLOPS_PER_PAIR_POINT / (pms * 1e-3) / 1e12
-            plain = {"path": "direct FP32 retarded sum, every pair (Kahan-compensated)",
+            plain = {"path": "direct FP32 retarded sum, every pair (every term compensated)",
                      "value": w.points / (pms / 1e3), "unit": UNIT, "ms_per_step": pms, "steps": nplain,
                      "speedup_of_ours": (w.points / (ms / K / 1e3)) / (w.points / (pms / 1e3)),
                      "pair_points_per_s": pp / (pms * 1e-3),

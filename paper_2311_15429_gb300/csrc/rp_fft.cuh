@@ -406,10 +406,10 @@ __host__ __device__ __forceinline__ void dft_b(float2 (&v)[B])
     else small_dft_c<B, INV>(v);
 }
 
-// Element (row p, line c) of a tile sits at T[p * SP + c * SC]: SP = 16 (or
-// more), SC = 1 for lines down the columns (rows of 16 consecutive lines), or
-// SP = 1 and SC odd for lines along the rows.  A half warp always serves the
-// 16 lines of one row, so both forms are free of bank conflicts.
+// Element (row p, line c) of a tile sits at T[p * SP + c * SC]; the kernels run
+// SP = 16, SC = 1, lines down the columns (rows of 16 consecutive lines; a half
+// warp always serves one row: no bank conflicts).  The other strides are the
+// host test's.
 //
 // Stage 1, task (c, n2): rows >= nin (and, with HALF, >= M/2) read as zero.
 template <int B, bool INV, bool HALF, int SP = 16, int SC = 1>

@@ -10,7 +10,7 @@ namespace rp {
 
 constexpr int kMaxDomains = 256;
 constexpr int kMaxFFT = 192;   // largest padded FFT length per axis
-constexpr int kThreads = 256;        // threads per block: ring push, register-blocked MAC
+constexpr int kThreads = 256;        // threads per block: ring push, general MAC
 constexpr int kPlaneThreads = 256;   // threads per block of the forward and inverse plane passes
 constexpr int kColumnThreads = 256;  // threads per block of the forward column pass
 constexpr int kTileY = 16;     // ky columns per block of the column passes

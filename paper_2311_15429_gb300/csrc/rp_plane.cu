@@ -25,16 +25,20 @@
 // keep every access free of bank conflicts.  Zero padding (inputs n >= M/2)
 // skips half of the first layer, cropping (outputs k >= M/2) half of the last.
 //
-// Shared memory per plane of n = M/2 and the blocks an SM holds: M = 96 39 KB
-// (5 forward, 4 inverse), M = 128 70 KB (3), M = 192 109 KB (2); the exchange of the y axis goes
-// in chunks of kx lines to keep it there.
+// Shared memory per plane of n = M/2 and the blocks an SM holds: M = 96 40 KB
+// forward (5) and 44 inverse (4), M = 128 70 and 73 KB (3), M = 192 111 KB (2);
+// the exchange of the y axis goes in chunks of kx lines to keep it there.
 // Per launch, before (tile and lane-shuffle forms) and now: 32 x 48^3 with far
-// pairs forward 111 -> 93 us, inverse 173 -> 117 (288 MB each: 42 us at the
-// copy rate); 8 x 64^3 92 -> 49 and 125 -> 63 (170 MB: 25 us); 3 x 96^3 100 ->
-// 68 and 188 -> 92 (198 MB: 29 us).  Half of the issue slots are used; what is
-// left is waits on the loads of T2 and on barriers at 24 to 27 warps per SM
-// (prefetching a round of lines, or fewer blocks with more registers, changed
-// nothing or lost).
+// pairs forward 111 -> 91 us, inverse 173 -> 112 (288 MB each: 42 us at the
+// copy rate); 8 x 64^3 92 -> 49 and 125 -> 61 (170 MB: 25 us); 3 x 96^3 100 ->
+// 67 and 188 -> 90 (198 MB: 29 us); 2 x 48^3 12.2 -> 11.3 and 13.7 -> 10.2.
+// Launches of about one wave are latency: 128 blocks of 64 points 6.7 -> 7.2
+// and 6.8 -> 7.5, 256 7.7 -> 7.1 and 7.6 -> 7.7, though the step of one 32^3
+// went from 22.8 to 19.8.  Below that, at 32 points, the forward pass has the
+// lane-shuffle form (kLanePlane32).  Half of the issue slots are used at many
+// waves; what is left is waits on the loads of T2 and on barriers at 24 to 27
+// warps per SM (prefetching a round of lines, or fewer blocks with more
+// registers, changed nothing or lost).
 #include <cuda_runtime.h>
 
 #include "rp_fft.cuh"
