@@ -1684,7 +1684,8 @@ rp_status overlapped_push(rp_ctx *ctx, int d0, int d1, const IoPtrs &in, cudaEve
 extern "C" {
 
 // Ground-state split, at a push of domains [d0, d1): on the first step keep
-// S(0) (pushed as it is, for the static potential); later, push Delta S.
+// S(0) (pushed as it is, for the static potential); later, push Delta S.  A
+// domain whose source another context owns has no slice.
 static rp_status split_inputs(rp_ctx *ctx, int d0, int d1, IoPtrs &in)
 {
     if (!ctx->split) return RP_OK;
@@ -1692,6 +1693,7 @@ static rp_status split_inputs(rp_ctx *ctx, int d0, int d1, IoPtrs &in)
     for (int d = d0; d < d1; ++d) {
         const long long N = ctx->doms[d].N;
         if (ctx->step == 0) {
+            if (!ctx->owned[d]) continue;
             RP_CUDA(ctx, cudaMemcpyAsync(ctx->ground[d], in.rho[d], N * sizeof(float), cudaMemcpyDeviceToDevice,
                                          ctx->stream));
             RP_CUDA(ctx, cudaMemcpyAsync(ctx->ground[d] + N, in.J[d], 3 * N * sizeof(float),
@@ -1703,6 +1705,7 @@ static rp_status split_inputs(rp_ctx *ctx, int d0, int d1, IoPtrs &in)
     if (ctx->step == 0) return RP_OK;
     RP_CUDA(ctx, launch_ground_delta(ctx->d_gdom, d0, d1, nblocks, in, ctx->stream));
     for (int d = d0; d < d1; ++d) {
+        if (!ctx->owned[d]) continue;
         in.rho[d] = ctx->delta[d];
         in.J[d] = ctx->delta[d] + ctx->doms[d].N;
     }

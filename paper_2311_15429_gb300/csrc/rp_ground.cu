@@ -16,8 +16,8 @@ namespace {
 
 constexpr int kGroundThreads = 256, kGroundChunk = 8 * kGroundThreads;
 
-// Every domain of the push in one launch (a launch of its own per domain, 2 to
-// 3 us each, was a tenth of the step of four 27^3 neighbours).
+// Every domain of the push that has a slice, in one launch (a launch of its own
+// per domain, 2 to 3 us each, was a tenth of the step of four 27^3 neighbours).
 __global__ void __launch_bounds__(kGroundThreads)
     k_ground_delta(const GroundDomain *__restrict__ doms, int d0, int d1, IoPtrs in)
 {
@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(kGroundThreads)
     }
     const GroundDomain D = doms[lo];
     const float *rho = in.rho[lo], *J = in.J[lo];
+    if (!rho) return;   // another context's source
     const long long base = (long long)(b - D.block0) * kGroundChunk + threadIdx.x;
     pdl_trigger();
     pdl_wait();   // the slices, and the last readers of delta
