@@ -1219,11 +1219,13 @@ rp_status rp_finalize(rp_ctx *ctx)
     if (const int most = ctx->plan_only ? kDirPlanLags : kDirMaxLags; max_nlag > most)
         return fail(ctx, RP_ERR_UNSUPPORTED, "direct pair lag window of " + std::to_string(max_nlag) +
                                                  " steps, above " + std::to_string(most));
-    // FP64 audit: every source keeps its raw slices as deep as its deepest pair reads
+    // FP64 audit: every owned source keeps its raw slices as deep as its deepest pair reads
     if (ctx->cfg.flags & RP_FLAG_AUDIT)
         for (int t = 0; t < nd; ++t)
             for (int s = 0; s < nd; ++s)
-                rdepth[s] = std::max(rdepth[s], ctx->pairs[(size_t)t * nd + s].lag_hi + 1 + (ctx->overlap ? 1 : 0));
+                if (ctx->owned[s])
+                    rdepth[s] = std::max(rdepth[s],
+                                         ctx->pairs[(size_t)t * nd + s].lag_hi + 1 + (ctx->overlap ? 1 : 0));
     ctx->dir_nlag = max_nlag;
     ctx->raw_block0.assign(nd + 1, 0);
     for (int d = 0; d < nd; ++d) {
