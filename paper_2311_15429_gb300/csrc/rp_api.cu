@@ -738,7 +738,7 @@ rp_status build_learned(rp_ctx *ctx, const std::vector<float> &weights, const st
 // in parts beside one another.  Without it (under a device budget, whose
 // planned bytes it would pass, or where the device has no room) a block runs
 // its targets' parts in turn: the same bits, only fewer blocks.  After every
-// other allocation of the plan.
+// other allocation of the plan but its own table.
 rp_status plan_direct(rp_ctx *ctx)
 {
     long long floats = 0;
@@ -765,7 +765,7 @@ rp_status plan_direct(rp_ctx *ctx)
         ctx->dir_blocks += D.blocks * (beside ? D.parts : 1);
         ctx->dir_sum_blocks += beside ? D.blocks : 0;
     }
-    return RP_OK;
+    return upload(ctx, &ctx->d_dtg, ctx->dtg);
 }
 
 // Launch-shape autotuning: time each consumer-warp variant of the TMA-fed MAC
@@ -1409,8 +1409,6 @@ rp_status rp_finalize(rp_ctx *ctx)
     if ((st = build_mix(ctx))) return st;
     if ((st = upload(ctx, &ctx->d_inv, ctx->inv))) return st;
     if ((st = upload(ctx, &ctx->d_entries, ctx->entries))) return st;
-    if ((st = plan_direct(ctx))) return st;
-    if ((st = upload(ctx, &ctx->d_dtg, ctx->dtg))) return st;
     if ((st = upload(ctx, &ctx->d_dpairs, ctx->dpairs))) return st;
     if ((st = upload(ctx, &ctx->d_raw, ctx->raw))) return st;
     RP_CUDA(ctx, open_kernel_smem_limits(max_optin));
@@ -1422,6 +1420,7 @@ rp_status rp_finalize(rp_ctx *ctx)
     // looked up here, at set-up, so that the module holding it is loaded (and
     // the array placed in device memory) now and not at that call's first use
     if ((st = noalloc_stage_address(ctx, &ctx->noalloc_stage))) return st;
+    if ((st = plan_direct(ctx))) return st;
     RP_CUDA(ctx, cudaDeviceSynchronize());
     if ((st = autotune_mac(ctx))) return st;
     ctx->finalized = true;
